@@ -722,20 +722,29 @@ struct CollCount {
   unsigned cand, coll, clip, inel;
 };
 
-template <typename T, bool GEN = true>
-__device__ __forceinline__ void collide_cell(const Params<T>& p, T* __restrict__ vx, T* __restrict__ vy,
-                             T* __restrict__ vz, T* __restrict__ ir, int n, uint32_t cell,
-                             uint32_t step, T* sgmax_ptr, uint32_t* owner, CollCount& cc) {
-  const int lane = threadIdx.x & 31;
-  if (!p.collisions || n < 2) return;
-  const T sgmax = *sgmax_ptr;
+// candidate pairs of the step (Iround of the NTC count); 0 where nothing collides
+template <typename T>
+__device__ __forceinline__ uint32_t ntc_candidates(const Params<T>& p, int n, uint32_t cell, uint32_t step, T sgmax) {
+  if (!p.collisions || n < 2) return 0u;
   const T vc = p.vol ? p.vol[cell] : p.vcell;  // the annulus's cells differ in volume
   const T xm = T(0.5) * T(n) * T(n - 1) * p.fnum * sgmax * p.dt / vc;
   Stream<T> sn(TAG_NTC, 0u, cell, step, p.k0, p.k1);
   const long long Mll = iround(xm, sn.u(0));
-  const uint32_t M = (uint32_t)(Mll < 0 ? 0 : Mll);
-  if (M == 0) return;
-  for (int q = lane; q < n; q += 32) owner[q] = OWNER_FREE;
+  return (uint32_t)(Mll < 0 ? 0 : Mll);
+}
+
+// The M candidates of a cell by the G lanes of one group (G = 32: the warp;
+// G = 8: four cells side by side, each with its own arguments).  The window
+// then holds up to G candidates; the result does not depend on its size.
+// Every lane of the warp calls it (M = 0 where a group has nothing to do).
+template <typename T, bool GEN, int G>
+__device__ __forceinline__ void collide_window(const Params<T>& p, T* __restrict__ vx, T* __restrict__ vy,
+                             T* __restrict__ vz, T* __restrict__ ir, int n, uint32_t cell,
+                             uint32_t step, T sgmax, uint32_t M, T* sgmax_ptr, uint32_t* owner, CollCount& cc) {
+  const int lane = threadIdx.x & 31, gl = lane & (G - 1);
+  const unsigned group = (G == 32) ? FULL : (((1u << (G & 31)) - 1u) << (lane & ~(G - 1)));
+  if (M != 0u)
+    for (int q = gl; q < n; q += G) owner[q] = OWNER_FREE;
   __syncwarp();
   T obs = T(0);
   uint32_t next = 0;
@@ -747,12 +756,12 @@ __device__ __forceinline__ void collide_cell(const Params<T>& p, T* __restrict__
   // lane still has a candidate to draw (later rounds run with few lanes)
   uint4 wpost = make_uint4(0u, 0u, 0u, 0u);
   const T fn = T(n), fn1 = T(n - 1);
-  const unsigned below = (1u << lane) - 1u;
+  const unsigned below = (1u << lane) - 1u;  // of the group, after the masking of freem
   // A lane keeps its candidate until it runs; free lanes take the next
   // candidates in order, so the window is always every unprocessed candidate
   // below `next` (which lane holds which does not matter).
   for (;;) {
-    const unsigned freem = __ballot_sync(FULL, !has);
+    const unsigned freem = __ballot_sync(FULL, !has) & group;
     if (!has) {
       const uint32_t kk = next + (uint32_t)__popc(freem & below);
       if (kk < M) {
@@ -844,12 +853,23 @@ __device__ __forceinline__ void collide_cell(const Params<T>& p, T* __restrict__
   }
   // (sigma g)_max takes the largest sigma g seen in the step
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int o = G / 2; o > 0; o >>= 1) {
     const T other = __shfl_xor_sync(FULL, obs, o);
     obs = other > obs ? other : obs;
   }
   __syncwarp();
-  if (lane == 0 && obs > sgmax) *sgmax_ptr = obs;
+  if (gl == 0 && M != 0u && obs > sgmax) *sgmax_ptr = obs;
+}
+
+// the candidates of one cell by its warp
+template <typename T, bool GEN = true>
+__device__ __forceinline__ void collide_cell(const Params<T>& p, T* __restrict__ vx, T* __restrict__ vy,
+                             T* __restrict__ vz, T* __restrict__ ir, int n, uint32_t cell,
+                             uint32_t step, T* sgmax_ptr, uint32_t* owner, CollCount& cc) {
+  const T sgmax = *sgmax_ptr;
+  const uint32_t M = ntc_candidates<T>(p, n, cell, step, sgmax);
+  if (M == 0u) return;
+  collide_window<T, GEN, 32>(p, vx, vy, vz, ir, n, cell, step, sgmax, M, sgmax_ptr, owner, cc);
 }
 
 // ---------------------------------------------------------------------------
@@ -952,20 +972,21 @@ __device__ __forceinline__ int halving_moment(int lane) {
   return ok ? j : -1;
 }
 
-template <int S, int OFF>
-__device__ __forceinline__ void halving_level(const float* in, float* out, int lane) {
+template <int S, int OFF, typename T>
+__device__ __forceinline__ void halving_level(const T* in, T* out, int lane) {
   constexpr int H = (S + 1) / 2;
   const bool up = (lane & OFF) != 0;
 #pragma unroll
   for (int i = 0; i < H; ++i) {
-    const float lo = in[i];
-    const float hi = (i + H < S) ? in[i + H] : 0.f;
+    const T lo = in[i];
+    const T hi = (i + H < S) ? in[i + H] : T(0);
     out[i] = (up ? hi : lo) + __shfl_xor_sync(FULL, up ? lo : hi, OFF);
   }
 }
 
-__device__ __forceinline__ float halving_sum17(const float* v, int lane) {
-  float a[9], b[5], c[3], d[2], e[1];
+template <typename T>
+__device__ __forceinline__ T halving_sum17(const T* v, int lane) {
+  T a[9], b[5], c[3], d[2], e[1];
   halving_level<17, 16>(v, a, lane);
   halving_level<9, 8>(a, b, lane);
   halving_level<5, 4>(b, c, lane);
@@ -979,14 +1000,15 @@ __device__ __forceinline__ float halving_sum17(const float* v, int lane) {
 // pre32 holds the lane's (stg, stc) loaded earlier).  With `flush` the staged
 // sum is folded into the compensated FP64 accumulators (pre: the lane's acc,
 // comp) and the staging pair is cleared.
-__device__ __forceinline__ void sample_accumulate(const float* __restrict__ vx, const float* __restrict__ vy,
-                                                  const float* __restrict__ vz, const float* __restrict__ ir, int n,
-                                                  float* s) {
+template <typename T>
+__device__ __forceinline__ void sample_accumulate(const T* __restrict__ vx, const T* __restrict__ vy,
+                                                  const T* __restrict__ vz, const T* __restrict__ ir, int n,
+                                                  T* s) {
   const int lane = threadIdx.x & 31;
   for (int q = lane; q < n; q += 32) {
-    const float a = vx[q], b = vy[q], c = vz[q], e = ir[q];
-    const float v2 = a * a + b * b + c * c;
-    s[0] += 1.f;
+    const T a = vx[q], b = vy[q], c = vz[q], e = ir[q];
+    const T v2 = a * a + b * b + c * c;
+    s[0] += T(1);
     s[1] += a;
     s[2] += b;
     s[3] += c;
@@ -1041,6 +1063,29 @@ __device__ __forceinline__ void sample_cell_staged(const float* __restrict__ vx,
   for (int q = 0; q < NMOM; ++q) s[q] = 0.f;
   sample_accumulate(vx, vy, vz, ir, n, s);
   sample_fold(halving_sum17(s, threadIdx.x & 31), mom, acc, comp, pre, stg, stc, pre32, flush);
+}
+
+// FP64 particles: this step's sums of one cell, added to the compensated
+// accumulators
+__device__ __forceinline__ void sample_cell_f64(const double* __restrict__ vx, const double* __restrict__ vy,
+                                                const double* __restrict__ vz, const double* __restrict__ ir, int n,
+                                                double* __restrict__ acc, double* __restrict__ comp) {
+  const int lane = threadIdx.x & 31, mom = halving_moment(lane);
+  double a = 0.0, cprev = 0.0;
+  if (mom >= 0) {
+    a = acc[mom];
+    cprev = comp[mom];
+  }
+  double s[NMOM];
+#pragma unroll
+  for (int q = 0; q < NMOM; ++q) s[q] = 0.0;
+  sample_accumulate(vx, vy, vz, ir, n, s);
+  const double v = halving_sum17(s, lane);
+  if (mom < 0) return;
+  const double t = a + v;
+  const double cmp = (fabs(a) >= fabs(v)) ? ((a - t) + v) : ((v - t) + a);
+  acc[mom] = t;
+  comp[mom] = cprev + cmp;
 }
 
 // one chunk of a cell's particles: its sums reduced across the warp (the

@@ -95,6 +95,7 @@ struct State {
   // atomics); fork after the previous launch, join before the next
   cudaStream_t side;
   cudaEvent_t ev_fork, ev_join;
+  bool count_clear;  // FP64 layout: the occupancies of the layout not in use are zero
   bool lost;  // FP64 annulus: freestream entries did not fit the workspace
 };
 

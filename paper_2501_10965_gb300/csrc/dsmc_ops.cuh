@@ -3,10 +3,11 @@
 // launch wrappers.  Included by one translation unit per precision.
 //
 // Two particle layouts:
-//  * FP64-deterministic: compact, cell-sorted arrays; each step runs
-//    move (one thread per particle) -> stable counting sort (one CTA) ->
-//    collide + sample (one warp per cell).  The event order equals the
-//    sequential definition, so results match a sequential implementation.
+//  * FP64-deterministic: compact, cell-sorted arrays; each step runs move
+//    (one thread per particle) -> scan of the new occupancies and lists of
+//    source slots per cell -> gather in slot order + collide + sample (one
+//    warp per cell).  The event order equals the sequential definition, so
+//    results match a sequential implementation.
 //  * FP32: each cell owns a padded bin; one fused kernel per step runs, per
 //    cell (one warp): stage the cell in shared memory, collide, sample, move,
 //    and append each particle to its new cell's bin in the other buffer
@@ -77,6 +78,68 @@ __device__ void cta_exclusive_scan(int n, F value, int32_t* out) {
   }
   if (threadIdx.x == 0) out[n] = carry;
   __syncthreads();
+}
+
+// ---------------------------------------------------------------------------
+// exclusive scan of v over the whole grid, CTA b the SCAN_CHUNK entries from b
+// SCAN_CHUNK: out[i] = sum_{k<i} v[k], out[n] = total.  A CTA adds up the
+// entries before its chunk itself (16-byte loads, from L2), so no CTA waits
+// for another and one launch does the scan; the redundant reads grow with
+// n^2 but are 13 MB at 160 000 cells.  Latency-bound; one CTA passing over
+// 160 000 cells in order took 107 us (three scans of a modification with
+// read-out of 32 M particles: 4.29 -> 3.99 ms in all).
+// total (may be null): the total is stored there too; flags (may be null):
+// bit 4 is set when the total exceeds capacity.
+// ---------------------------------------------------------------------------
+constexpr int SCAN_CHUNK = 4096;
+static __global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict__ v, int n, int32_t* __restrict__ out,
+                                                      int32_t* __restrict__ total, int32_t* __restrict__ flags,
+                                                      long long capacity) {
+  __shared__ int32_t s_pre[32], s_own[32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int base = blockIdx.x * SCAN_CHUNK;
+  int32_t pre = 0;
+  const int4* v4 = reinterpret_cast<const int4*>(v);
+  for (int i = threadIdx.x; i < base / 4; i += 1024) {
+    const int4 q = v4[i];
+    pre += (q.x + q.y) + (q.z + q.w);
+  }
+  const int i0 = base + 4 * (int)threadIdx.x;
+  int32_t e[4], t = 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    e[j] = (i0 + j < n) ? v[i0 + j] : 0;
+    t += e[j];
+  }
+  int32_t x = t;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int32_t y = __shfl_up_sync(FULL, x, o);
+    if (lane >= o) x += y;
+  }
+  pre = __reduce_add_sync(FULL, pre);
+  if (lane == 31) {
+    s_pre[warp] = pre;
+    s_own[warp] = x;
+  }
+  __syncthreads();
+  const int32_t before = __reduce_add_sync(FULL, s_pre[lane] + (lane < warp ? s_own[lane] : 0));
+  int32_t run = before + x - t;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    if (i0 + j < n) out[i0 + j] = run;
+    run += e[j];
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 1023) {
+    out[n] = run;
+    if (total) *total = run;
+    if (flags && (long long)run > capacity) atomicOr(flags, 4);
+  }
+}
+
+inline void launch_scan(const int32_t* v, int n, int32_t* out, cudaStream_t st, int32_t* total = nullptr,
+                        int32_t* flags = nullptr, long long capacity = 0) {
+  k_scan<<<(n + SCAN_CHUNK - 1) / SCAN_CHUNK, 1024, 0, st>>>(v, n, out, total, flags, capacity);
 }
 
 __device__ __forceinline__ int32_t bin_cap_of(int32_t count, double slack) {
@@ -174,43 +237,75 @@ static __global__ void k_layout_uniform(int ncells, int32_t cap, int32_t* start)
 }
 
 // ---------------------------------------------------------------------------
-// FP64-deterministic layout: move, stable sort, collide + sample
+// FP64-deterministic layout.  A step is move (+ a count per new cell) -> scan
+// of the counts -> each cell's list of source slots -> per cell: order the
+// list, gather the particles, collide, sample, write.  The particles of a
+// cell follow in the order of their slots before the move, as a stable sort
+// by cell would leave them; only the lists, not the particles, pass through
+// the unordered atomics, and the ascending slot numbers restore the order.
 // ---------------------------------------------------------------------------
+
+// one arrival per lane with key k >= 0 (k < 0: none): its number within the
+// cell, one atomic per group of lanes with the same cell (the particles are
+// sorted by cell before the move, so a warp meets few cells)
+__device__ __forceinline__ int32_t cell_arrival(int32_t* __restrict__ cnt, int k) {
+  const int lane = threadIdx.x & 31;
+  const unsigned peers = __match_any_sync(FULL, k);
+  const int leader = __ffs(peers) - 1;
+  int32_t b = 0;
+  if (k >= 0 && lane == leader) b = atomicAdd(&cnt[k], __popc(peers));
+  b = __shfl_sync(FULL, b, leader);
+  return b + __popc(peers & ((1u << lane) - 1u));
+}
+
+// move; key[s] = the new cell (-1: left the annulus), arr[s] = the arrival
+// number in it, cnt = the new occupancies (zero before)
 template <typename T, int DIM, bool BATCH, bool ANN>
 __global__ void __launch_bounds__(256) k_move_det(const __grid_constant__ Params<T> pk, Cases<T> cases, PBuf<T> b,
                                                   const int32_t* __restrict__ cellof,
                                                   const int32_t* __restrict__ start, int n,
                                                   uint32_t step, int32_t* __restrict__ key,
+                                                  int32_t* __restrict__ arr, int32_t* __restrict__ cnt,
                                                   double* __restrict__ tally_g,
                                                   unsigned long long* __restrict__ stats) {
   __shared__ T s_tally[20];
   if (threadIdx.x < 20) s_tally[threadIdx.x] = T(0);
   __syncthreads();
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-    const int c = cellof[s];
-    const int cs = BATCH ? cases.cell_case[c] : 0;
-    const Params<T>& p = BATCH ? cases.p[cs] : pk;
-    const int c0 = BATCH ? cases.cell0[cs] : 0;
-    T x = b.x[s], y = b.y[s], vx = b.vx[s], vy = b.vy[s], vz = b.vz[s], ir = b.ir[s];
-    bool in = true;
-    if constexpr (ANN)
-      in = fly_ann<T, true>(p, x, y, vx, vy, vz, ir, TAG_WALL, (uint32_t)(s - start[c]), (uint32_t)c, step, 0u, p.dt,
-                            s_tally, stats + ST_HITS, stats + ST_MAXHIT);
-    else
-      fly<T, DIM, true>(p, x, y, vx, vy, vz, ir, (uint32_t)(s - start[c]), (uint32_t)(c - c0), step, s_tally,
-                        stats + ST_HITS, stats + ST_MAXHIT);
-    b.x[s] = x;
-    b.y[s] = y;
-    b.vx[s] = vx;
-    b.vy[s] = vy;
-    b.vz[s] = vz;
-    b.ir[s] = ir;
-    if constexpr (ANN) {
-      // a particle that left keeps key -1: the sort drops it
-      key[s] = in ? cell_of_ann<T>(p, x, y) : -1;
-      if (!in) atomicAdd(stats + ST_OUT, 1ull);
-    } else {
-      key[s] = c0 + cell_of<T, DIM>(p, x, y);
+  const int lane = threadIdx.x & 31;
+  for (int s0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); s0 < n; s0 += gridDim.x * blockDim.x) {
+    const int s = s0 + lane;
+    int k = -1;
+    if (s < n) {
+      const int c = cellof[s];
+      const int cs = BATCH ? cases.cell_case[c] : 0;
+      const Params<T>& p = BATCH ? cases.p[cs] : pk;
+      const int c0 = BATCH ? cases.cell0[cs] : 0;
+      T x = b.x[s], y = b.y[s], vx = b.vx[s], vy = b.vy[s], vz = b.vz[s], ir = b.ir[s];
+      bool in = true;
+      if constexpr (ANN)
+        in = fly_ann<T, true>(p, x, y, vx, vy, vz, ir, TAG_WALL, (uint32_t)(s - start[c]), (uint32_t)c, step, 0u, p.dt,
+                              s_tally, stats + ST_HITS, stats + ST_MAXHIT);
+      else
+        fly<T, DIM, true>(p, x, y, vx, vy, vz, ir, (uint32_t)(s - start[c]), (uint32_t)(c - c0), step, s_tally,
+                          stats + ST_HITS, stats + ST_MAXHIT);
+      b.x[s] = x;
+      b.y[s] = y;
+      b.vx[s] = vx;
+      b.vy[s] = vy;
+      b.vz[s] = vz;
+      b.ir[s] = ir;
+      if constexpr (ANN) {
+        // a particle that left keeps key -1: no list holds it
+        k = in ? cell_of_ann<T>(p, x, y) : -1;
+        if (!in) atomicAdd(stats + ST_OUT, 1ull);
+      } else {
+        k = c0 + cell_of<T, DIM>(p, x, y);
+      }
+    }
+    const int32_t a = cell_arrival(cnt, k);
+    if (s < n) {
+      key[s] = k;
+      arr[s] = a;
     }
   }
   __syncthreads();
@@ -218,57 +313,89 @@ __global__ void __launch_bounds__(256) k_move_det(const __grid_constant__ Params
     atomicAdd(tally_g + threadIdx.x, (double)s_tally[threadIdx.x]);
 }
 
-// Stable counting sort by key (one CTA of 1024 threads): histogram, scan,
-// then one warp assigns destinations 32 slots at a time in slot order (ties
-// keep their order), then every thread scatters.  Tin -> Tout conversion.
-template <typename Tin, typename Tout>
-__global__ void __launch_bounds__(1024) k_sort_stable(const Tin* __restrict__ ix, const Tin* __restrict__ iy,
-                                                      const Tin* __restrict__ ivx, const Tin* __restrict__ ivy,
-                                                      const Tin* __restrict__ ivz, const Tin* __restrict__ iir,
-                                                      PBuf<Tout> o, const int32_t* __restrict__ key, int n,
-                                                      int ncells, int32_t* __restrict__ start_out,
-                                                      int32_t* __restrict__ count_out,
-                                                      int32_t* __restrict__ fill,
-                                                      int32_t* __restrict__ dest,
-                                                      int32_t* __restrict__ cellof_out) {
-  for (int c = threadIdx.x; c < ncells; c += blockDim.x) count_out[c] = 0;
-  __syncthreads();
-  for (int s = threadIdx.x; s < n; s += blockDim.x)
-    if (key[s] >= 0) atomicAdd(&count_out[key[s]], 1);  // key -1: the particle left
-  __syncthreads();
-  cta_exclusive_scan(ncells, [&](int i) { return count_out[i]; }, start_out);
-  for (int c = threadIdx.x; c < ncells; c += blockDim.x) fill[c] = start_out[c];
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    const int lane = threadIdx.x;
-    for (int base = 0; base < n; base += 32) {
-      const int s = base + lane;
-      const int k = (s < n) ? key[s] : -1;
-      const unsigned peers = __match_any_sync(FULL, k);
-      const int leader = __ffs(peers) - 1;
+// arrival numbers and occupancies of imported particles
+static __global__ void k_arrivals(const int32_t* __restrict__ key, int n, int32_t* __restrict__ cnt,
+                                  int32_t* __restrict__ arr) {
+  const int lane = threadIdx.x & 31;
+  for (int s0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); s0 < n; s0 += gridDim.x * blockDim.x) {
+    const int s = s0 + lane;
+    const int32_t a = cell_arrival(cnt, (s < n) ? key[s] : -1);
+    if (s < n) arr[s] = a;
+  }
+}
+
+// the lists of source slots, in order of arrival
+static __global__ void k_det_lists(const int32_t* __restrict__ key, const int32_t* __restrict__ arr, int n,
+                                   const int32_t* __restrict__ start, int32_t* __restrict__ list) {
+  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
+    const int k = key[s];
+    if (k >= 0) list[start[k] + arr[s]] = s;
+  }
+}
+
+// scan and lists in one CTA, for few particles and cells (one launch less)
+static __global__ void __launch_bounds__(1024) k_det_lists_small(const int32_t* __restrict__ cnt, int ncells,
+                                                                 const int32_t* __restrict__ key,
+                                                                 const int32_t* __restrict__ arr, int n,
+                                                                 int32_t* __restrict__ start,
+                                                                 int32_t* __restrict__ list) {
+  cta_exclusive_scan(ncells, [&](int i) { return cnt[i]; }, start);
+  for (int s = threadIdx.x; s < n; s += 1024) {
+    const int k = key[s];
+    if (k >= 0) list[start[k] + arr[s]] = s;
+  }
+}
+
+// Ascending order of a cell's list that does not fit the tile: one warp,
+// least significant 8 bits first (list <-> tmp, both in global memory), hist
+// 256 words of shared memory; returns the buffer that holds the result.
+// nbits covers the largest slot number.
+__device__ inline int32_t* sort_list_global(int32_t* list, int32_t* tmp, int n, int nbits, int32_t* hist) {
+  const int lane = threadIdx.x & 31;
+  for (int sh = 0; sh < nbits; sh += 8) {
+    for (int d = lane; d < 256; d += 32) hist[d] = 0;
+    __syncwarp();
+    for (int q = lane; q < n; q += 32) atomicAdd(&hist[(list[q] >> sh) & 255], 1);
+    __syncwarp();
+    int32_t v[8], t = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      v[j] = hist[8 * lane + j];
+      t += v[j];
+    }
+    int32_t x = t;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(FULL, x, o);
+      if (lane >= o) x += y;
+    }
+    x -= t;
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      hist[8 * lane + j] = x;
+      x += v[j];
+    }
+    __syncwarp();
+    for (int q0 = 0; q0 < n; q0 += 32) {
+      const int q = q0 + lane;
+      const int32_t s = (q < n) ? list[q] : -1;
+      const int d = (q < n) ? ((s >> sh) & 255) : -1;
+      const unsigned peers = __match_any_sync(FULL, d);
       const int rank = __popc(peers & ((1u << lane) - 1u));
-      int b = 0;
-      if (s < n && k >= 0 && lane == leader) {
-        b = fill[k];
-        fill[k] = b + __popc(peers);
+      const int32_t b = (d >= 0) ? hist[d] : 0;
+      __syncwarp();
+      if (d >= 0) {
+        tmp[b + rank] = s;
+        if (rank == 0) hist[d] = b + __popc(peers);
       }
-      b = __shfl_sync(FULL, b, leader);
-      if (s < n) dest[s] = (k >= 0) ? b + rank : -1;
       __syncwarp();
     }
+    int32_t* o = list;
+    list = tmp;
+    tmp = o;
   }
-  __syncthreads();
-  for (int s = threadIdx.x; s < n; s += blockDim.x) {
-    const int d = dest[s];
-    if (d < 0) continue;
-    o.x[d] = (Tout)ix[s];
-    o.y[d] = (Tout)iy[s];
-    o.vx[d] = (Tout)ivx[s];
-    o.vy[d] = (Tout)ivy[s];
-    o.vz[d] = (Tout)ivz[s];
-    o.ir[d] = (Tout)iir[s];
-    if (cellof_out) cellof_out[d] = key[s];
-  }
+  return list;
 }
 
 // ---------------------------------------------------------------------------
@@ -319,11 +446,12 @@ __device__ __forceinline__ bool inflow_particle(const Params<double>& p, int k, 
 // FP64 layout, one CTA: a scan gives each face its run of slots after the n
 // moved particles, so that new particles follow face by face and, within a
 // face, in draw order (the sequential algorithm's order).  One that ends
-// outside keeps key -1 (the sort drops it).  cnt, off: nx and nx + 1 ints;
-// off[nx] is the number of slots used.
+// outside keeps key -1 (no cell's list holds it).  cnt, off: nx and nx + 1
+// ints; off[nx] is the number of slots used.  cell_cnt, arr: as k_move_det's.
 template <typename T>
 __global__ void __launch_bounds__(1024) k_inject_det(const __grid_constant__ Params<double> p, PBuf<T> b,
-                                                     int32_t* __restrict__ key, int n, long long capacity,
+                                                     int32_t* __restrict__ key, int32_t* __restrict__ arr,
+                                                     int32_t* __restrict__ cell_cnt, int n, long long capacity,
                                                      uint32_t step, int32_t* __restrict__ cnt,
                                                      int32_t* __restrict__ off, int32_t* __restrict__ flags,
                                                      double* __restrict__ tally_g,
@@ -352,7 +480,9 @@ __global__ void __launch_bounds__(1024) k_inject_det(const __grid_constant__ Par
       b.vy[slot] = (T)vy;
       b.vz[slot] = (T)vz;
       b.ir[slot] = (T)ir;
-      key[slot] = in ? cell_of_ann<double>(p, x, y) : -1;
+      const int kc = in ? cell_of_ann<double>(p, x, y) : -1;
+      key[slot] = kc;
+      if (kc >= 0) arr[slot] = atomicAdd(&cell_cnt[kc], 1);
       if (in) ++nin;  // one that ends outside never entered
     }
   }
@@ -543,6 +673,166 @@ __device__ __forceinline__ void flush_counts(const CollCount& cc, unsigned* s_cn
     atomicAdd(s_cnt + 2, c);
     atomicAdd(s_cnt + 3, d);
   }
+}
+
+// FP64 layout, one warp per cell: order the cell's list of source slots,
+// gather its particles (positions straight to the output, velocities and
+// energies to shared memory; cells above `tile` particles work in the output
+// arrays), run NTC collisions and/or sampling, write.  flags: 1 collide, 2
+// sample (0: a plain sort).  cnt_old, the occupancies of the layout left
+// behind, are cleared for the next step's count.
+//
+// The FP64 pipe bounds it (one warp instruction per 16 cycles and SM, however
+// many lanes are active) and a cell has few candidates, so with 8 warps per
+// CTA one warp takes the candidates of four cells, 8 lanes each, when none of
+// them has more than GROUP_MAX_M: a quarter of the instructions.  GROUP_MAX_M:
+// above it the 8-lane window's rounds outnumber what the sharing saves.  With
+// one warp per CTA (few cells: every cell has an SM's pipe to itself) the
+// cell's own warp takes them.
+constexpr uint32_t GROUP_MAX_M = 24u;
+template <typename T, bool BATCH>
+__global__ void __launch_bounds__(WPB * 32) k_det_cells(const __grid_constant__ Params<T> pk, Cases<T> cases,
+                                                        int ncells, const T* __restrict__ ix,
+                                                        const T* __restrict__ iy, const T* __restrict__ ivx,
+                                                        const T* __restrict__ ivy, const T* __restrict__ ivz,
+                                                        const T* __restrict__ iir, PBuf<T> b,
+                                                        const int32_t* __restrict__ start,
+                                                        const int32_t* __restrict__ count,
+                                                        int32_t* __restrict__ cnt_old, int32_t* __restrict__ list,
+                                                        int nbits, int32_t* __restrict__ cellof,
+                                                        T* __restrict__ sgmax, double* __restrict__ acc,
+                                                        double* __restrict__ comp, uint32_t* __restrict__ owner_g,
+                                                        uint32_t step, int flags, int tile,
+                                                        unsigned long long* __restrict__ stats) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ unsigned s_cnt[4];
+  __shared__ uint32_t s_m[WPB];
+  __shared__ int s_n[WPB];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  if (threadIdx.x < 4) s_cnt[threadIdx.x] = 0;
+  __syncthreads();
+  const int cell = blockIdx.x * nw + warp;
+  const bool live = cell < ncells;
+  auto tile_of = [&](int w) { return reinterpret_cast<T*>(smem) + (size_t)w * tile * 4; };
+  auto owner_of = [&](int w) {
+    return reinterpret_cast<uint32_t*>(smem + (size_t)nw * tile * 4 * sizeof(T)) + (size_t)w * tile;
+  };
+  const int cs = (BATCH && live) ? cases.cell_case[cell] : 0;
+  const Params<T>& p = BATCH ? cases.p[cs] : pk;
+  const int lcell = cell - (BATCH ? cases.cell0[cs] : 0);
+  int base = 0, n = 0;
+  uint32_t M = 0;
+  T sg = T(0);
+  T *vx = tile_of(warp), *vy = vx + tile, *vz = vx + 2 * tile, *ir = vx + 3 * tile;
+  uint32_t* own = owner_of(warp);
+  bool staged = true;
+  if (live) {
+    base = start[cell];
+    n = count[cell];
+    if (lane == 0 && cnt_old) cnt_old[cell] = 0;
+    staged = n <= tile;
+    const int32_t* order;
+    if (staged) {
+      // slots are distinct: a slot's place is the number of smaller ones
+      constexpr int PER = TILE_MAX_OF<T> / 32;
+      int32_t* sl = reinterpret_cast<int32_t*>(own);
+      const int n4 = (n + 3) & ~3;  // tile is a multiple of 32
+      int32_t e[PER];
+      for (int q = lane; q < n4; q += 32) sl[q] = (q < n) ? list[base + q] : 0x7fffffff;
+      __syncwarp();
+      int32_t r[PER];
+#pragma unroll
+      for (int j = 0; j < PER; ++j) {
+        e[j] = (lane + 32 * j < n) ? sl[lane + 32 * j] : 0x7fffffff;
+        r[j] = 0;
+      }
+      for (int q = 0; q < n4; q += 4) {
+        const int4 o = *reinterpret_cast<const int4*>(sl + q);
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+          if (32 * j >= n) break;
+          r[j] += (o.x < e[j]) + (o.y < e[j]) + (o.z < e[j]) + (o.w < e[j]);
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < PER; ++j)
+        if (lane + 32 * j < n) sl[r[j]] = e[j];
+      __syncwarp();
+      order = sl;
+    } else {
+      vx = b.vx + base;
+      vy = b.vy + base;
+      vz = b.vz + base;
+      ir = b.ir + base;
+      own = owner_g + base;
+      order = sort_list_global(list + base, reinterpret_cast<int32_t*>(owner_g) + base, n, nbits,
+                               reinterpret_cast<int32_t*>(tile_of(warp)));
+    }
+    for (int q = lane; q < n; q += 32) {
+      const int s = order[q];
+      const T x = ix[s], y = iy[s], a = ivx[s], bb = ivy[s], c = ivz[s], e = iir[s];
+      b.x[base + q] = x;
+      b.y[base + q] = y;
+      vx[q] = a;
+      vy[q] = bb;
+      vz[q] = c;
+      ir[q] = e;
+      cellof[base + q] = cell;
+    }
+    __syncwarp();
+    if (flags & 1) {
+      sg = sgmax[cell];
+      M = ntc_candidates<T>(p, n, (uint32_t)lcell, step, sg);
+    }
+  }
+  if (flags & 1) {
+    CollCount cc{0, 0, 0, 0};
+    bool grouped = false;
+    if (nw == WPB) {
+      if (lane == 0) {
+        s_m[warp] = staged ? M : GROUP_MAX_M + 1u;
+        s_n[warp] = n;
+      }
+      __syncthreads();
+      uint32_t mm = 0;
+#pragma unroll
+      for (int w = 0; w < WPB; ++w) mm = max(mm, s_m[w]);
+      grouped = mm <= GROUP_MAX_M;
+      if (grouped && warp < WPB / 4) {
+        // cells 4 warp .. 4 warp + 3 of the CTA, 8 lanes each
+        const int w = 4 * warp + (lane >> 3), c = blockIdx.x * WPB + w;
+        const bool has = c < ncells;
+        const int gcs = (BATCH && has) ? cases.cell_case[c] : 0;
+        const Params<T>& gp = BATCH ? cases.p[gcs] : pk;
+        T* gv = tile_of(w);
+        collide_window<T, true, 8>(gp, gv, gv + tile, gv + 2 * tile, gv + 3 * tile, s_n[w],
+                                   (uint32_t)(c - (BATCH ? cases.cell0[gcs] : 0)), step, has ? sgmax[c] : T(0),
+                                   has ? s_m[w] : 0u, sgmax + (has ? c : 0), owner_of(w), cc);
+        flush_counts<T>(cc, s_cnt);
+      }
+      __syncthreads();
+    }
+    if (!grouped && live && M != 0u) {
+      collide_window<T, true, 32>(p, vx, vy, vz, ir, n, (uint32_t)lcell, step, sg, M, sgmax + cell, own, cc);
+      flush_counts<T>(cc, s_cnt);
+      __syncwarp();
+    }
+  }
+  if (live) {
+    if (flags & 2)
+      sample_cell_f64(vx, vy, vz, ir, n, acc + (size_t)cell * NMOM, comp + (size_t)cell * NMOM);
+    if (staged) {
+      for (int q = lane; q < n; q += 32) {
+        b.vx[base + q] = vx[q];
+        b.vy[base + q] = vy[q];
+        b.vz[base + q] = vz[q];
+        b.ir[base + q] = ir[q];
+      }
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 4 && s_cnt[threadIdx.x]) atomicAdd(stats + threadIdx.x, (unsigned long long)s_cnt[threadIdx.x]);
 }
 
 // One warp per cell: stage the cell's velocities and rotational energies in
@@ -1200,11 +1490,6 @@ __global__ void k_rebin_ovf(const Ovf ov, int ovf_cap, PBuf<float> out, const in
 // ---------------------------------------------------------------------------
 // export / import
 // ---------------------------------------------------------------------------
-static __global__ void __launch_bounds__(1024) k_scan_counts(const int32_t* __restrict__ cnt, int ncells,
-                                                      int32_t* __restrict__ out) {
-  cta_exclusive_scan(ncells, [&](int i) { return cnt[i]; }, out);
-}
-
 template <typename T>
 __global__ void __launch_bounds__(WPB * 32) k_export(PBuf<T> b, const int32_t* __restrict__ start,
                                                      const int32_t* __restrict__ cnt,
@@ -1340,16 +1625,6 @@ static __global__ void k_dig_counts(const CellParams* __restrict__ cps, const in
       if (c64) atomicAdd(reinterpret_cast<unsigned long long*>(flags + 4), c64);
       if (k64) atomicAdd(reinterpret_cast<unsigned long long*>(flags + 6), k64);
     }
-  }
-}
-
-static __global__ void __launch_bounds__(1024) k_scan_caps(const int32_t* __restrict__ caps, int ncells,
-                                                    long long capacity, int32_t* __restrict__ start_out,
-                                                    int32_t* __restrict__ flags) {
-  cta_exclusive_scan(ncells, [&](int i) { return caps[i]; }, start_out);
-  if (threadIdx.x == 0) {
-    flags[1] = start_out[ncells];
-    if ((long long)start_out[ncells] > capacity) atomicOr(flags, 4);
   }
 }
 
@@ -1613,64 +1888,93 @@ static void launch_collide_sample(const Params<T>& p, State<T>& s, int ncells, c
       p, s.cases, ncells, b, start, count, s.sgmax, s.acc, s.comp, s.owner, step, flags, s.tile, s.stats, stg, stc);
 }
 
+// up to this many slots and cells: scan and lists in one single-CTA launch
+// (one launch less, about 3 us, where a CTA's 1024 threads take at most 16
+// slots each).  A step of 10 000 particles on 100 cells: 138 us with the
+// single-CTA stable sort, 71 us with these kernels; of 500 000 on 10 000
+// cells: 5.1 ms, of which 4.0 in that sort, and 1.0 ms.
+constexpr int DET_SMALL = 16384;
+
+// FP64 layout: particles with cells `key` and arrival numbers `arr` (n slots
+// of the six input arrays, occupancies s.count[olay]) into buffer `other`,
+// layout olay; then flags as k_det_cells.  clear: the occupancies of the
+// layout left behind are cleared (they are not read again).
+template <typename T>
+static void det_cells(const Params<T>& p, State<T>& s, int n, const T* x, const T* y, const T* vx, const T* vy,
+                      const T* vz, const T* ir, int other, int olay, uint32_t step, int flags, bool clear,
+                      cudaStream_t st) {
+  const int ncells = s.ncells;
+  int32_t* list = s.scratch_i;
+  if (n <= DET_SMALL && ncells <= DET_SMALL) {
+    k_det_lists_small<<<1, 1024, 0, st>>>(s.count[olay], ncells, s.key, s.dest, n, s.start[olay], list);
+  } else {
+    launch_scan(s.count[olay], ncells, s.start[olay], st);
+    if (n > 0) k_det_lists<<<grid_for(n, 256), 256, 0, st>>>(s.key, s.dest, n, s.start[olay], list);
+  }
+  int nbits = 1;
+  while (nbits < 31 && (n >> nbits) != 0) ++nbits;
+  // up to two cells per SM: one warp per CTA spreads them over the SMs
+  const int nw = ncells <= 2 * 152 ? 1 : WPB;
+  const int blocks = (ncells + nw - 1) / nw;
+  const size_t sm = (size_t)nw * s.tile * (4 * sizeof(T) + sizeof(uint32_t));
+  int32_t* old = clear ? s.count[olay ^ 1] : nullptr;
+  if (s.batch)
+    k_det_cells<T, true><<<blocks, nw * 32, sm, st>>>(p, s.cases, ncells, x, y, vx, vy, vz, ir, s.buf[other],
+                                                      s.start[olay], s.count[olay], old, list, nbits, s.cellof,
+                                                      s.sgmax, s.acc, s.comp, s.owner, step, flags, s.tile, s.stats);
+  else
+    k_det_cells<T, false><<<blocks, nw * 32, sm, st>>>(p, s.cases, ncells, x, y, vx, vy, vz, ir, s.buf[other],
+                                                       s.start[olay], s.count[olay], old, list, nbits, s.cellof,
+                                                       s.sgmax, s.acc, s.comp, s.owner, step, flags, s.tile, s.stats);
+}
+
 template <typename T>
 void Ops<T>::step_det(const Params<T>& p, State<T>& s, int& cur, int& lay, uint32_t step, int do_sample,
                       cudaStream_t st) {
-  const int n = s.nparticles;
-  const int ncells = s.ncells;
-  const int other = cur ^ 1, olay = lay ^ 1;
-  if (n > 0) {
-    const int g = grid_for(n, 256);
-    if (p.mesh == 1) {
-      k_move_det<T, 2, false, true><<<g, 256, 0, st>>>(p, s.cases, s.buf[cur], s.cellof, s.start[lay], n, step,
-                                                       s.key, s.tally, s.stats);
-    } else if (p.dim == 1) {
-      if (s.batch)
-        k_move_det<T, 1, true, false><<<g, 256, 0, st>>>(p, s.cases, s.buf[cur], s.cellof, s.start[lay], n, step,
-                                                         s.key, s.tally, s.stats);
-      else
-        k_move_det<T, 1, false, false><<<g, 256, 0, st>>>(p, s.cases, s.buf[cur], s.cellof, s.start[lay], n, step,
-                                                          s.key, s.tally, s.stats);
-    } else {
-      if (s.batch)
-        k_move_det<T, 2, true, false><<<g, 256, 0, st>>>(p, s.cases, s.buf[cur], s.cellof, s.start[lay], n, step,
-                                                         s.key, s.tally, s.stats);
-      else
-        k_move_det<T, 2, false, false><<<g, 256, 0, st>>>(p, s.cases, s.buf[cur], s.cellof, s.start[lay], n, step,
-                                                          s.key, s.tally, s.stats);
+  if constexpr (sizeof(T) == 8) {
+    const int n = s.nparticles;
+    const int other = cur ^ 1, olay = lay ^ 1;
+    int32_t* cnt = s.count[olay];
+    if (!s.count_clear) cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)s.ncells, st);
+    if (n > 0) {
+      const int g = grid_for(n, 256);
+#define DSMC_MOVE_DET(D, B, A)                                                                                  \
+  k_move_det<T, D, B, A><<<g, 256, 0, st>>>(p, s.cases, s.buf[cur], s.cellof, s.start[lay], n, step, s.key, s.dest, \
+                                            cnt, s.tally, s.stats)
+      if (p.mesh == 1) DSMC_MOVE_DET(2, false, true);
+      else if (p.dim == 1 && s.batch) DSMC_MOVE_DET(1, true, false);
+      else if (p.dim == 1) DSMC_MOVE_DET(1, false, false);
+      else if (s.batch) DSMC_MOVE_DET(2, true, false);
+      else DSMC_MOVE_DET(2, false, false);
+#undef DSMC_MOVE_DET
     }
+    int ntot = n;
+    if (p.mesh == 1) {
+      // annulus: freestream entry after the moved particles; the host learns
+      // how many slots it used (particles that left are on no cell's list)
+      k_inject_det<T><<<1, 1024, 0, st>>>(s.pinj, s.buf[cur], s.key, s.dest, cnt, n, (long long)s.capacity, step,
+                                          s.nt, s.tmp2, s.flags, s.tally, s.stats);
+      int32_t add = 0;
+      cudaMemcpyAsync(&add, s.tmp2 + p.nx, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+      cudaStreamSynchronize(st);
+      const long long tot = (long long)n + add;
+      ntot = (int)(tot < s.capacity ? tot : s.capacity);
+      if (tot > s.capacity) s.lost = true;  // entries beyond the workspace were not written
+    }
+    const PBuf<T>& a = s.buf[cur];
+    det_cells<T>(p, s, ntot, a.x, a.y, a.vx, a.vy, a.vz, a.ir, other, olay, step, 1 | (do_sample ? 2 : 0), true, st);
+    s.count_clear = true;
+    cur = other;
+    lay = olay;
+    if (p.mesh == 1) {
+      int32_t kept = 0;
+      cudaMemcpyAsync(&kept, s.start[lay] + s.ncells, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
+      cudaStreamSynchronize(st);
+      s.nparticles = kept;
+    }
+  } else {
+    (void)p; (void)s; (void)cur; (void)lay; (void)step; (void)do_sample; (void)st;
   }
-  int ntot = n;
-  if (p.mesh == 1) {
-    // annulus: freestream entry after the moved particles; the host learns
-    // how many slots it used, the sort drops the particles that left
-    k_inject_det<T><<<1, 1024, 0, st>>>(s.pinj, s.buf[cur], s.key, n, (long long)s.capacity, step, s.nt, s.tmp2,
-                                        s.flags, s.tally, s.stats);
-    int32_t add = 0;
-    cudaMemcpyAsync(&add, s.tmp2 + p.nx, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-    cudaStreamSynchronize(st);
-    const long long tot = (long long)n + add;
-    ntot = (int)(tot < s.capacity ? tot : s.capacity);
-    if (tot > s.capacity) s.lost = true;  // entries beyond the workspace were not written
-  }
-  const PBuf<T>& a = s.buf[cur];
-  k_sort_stable<T, T><<<1, 1024, 0, st>>>(a.x, a.y, a.vx, a.vy, a.vz, a.ir, s.buf[other], s.key, ntot, ncells,
-                                          s.start[olay], s.count[olay], s.tmp2, s.dest, s.cellof);
-  cur = other;
-  lay = olay;
-  if (p.mesh == 1) {
-    int32_t kept = 0;
-    cudaMemcpyAsync(&kept, s.start[lay] + ncells, sizeof(int32_t), cudaMemcpyDeviceToHost, st);
-    cudaStreamSynchronize(st);
-    s.nparticles = kept;
-  }
-  const int flags = 1 | (do_sample ? 2 : 0);
-  if (s.batch)
-    launch_collide_sample<T, true>(p, s, ncells, s.buf[cur], s.start[lay], s.count[lay], step, flags, nullptr,
-                                   nullptr, st);
-  else
-    launch_collide_sample<T, false>(p, s, ncells, s.buf[cur], s.start[lay], s.count[lay], step, flags, nullptr,
-                                    nullptr, st);
 }
 
 template <typename T>
@@ -1840,7 +2144,7 @@ void Ops<T>::export_particles(const Params<T>& p, State<T>& s, int cur, int lay,
                               double* vy, double* vz, double* ir, int32_t* cell, cudaStream_t st) {
   (void)p;
   const int cntlay = (sizeof(T) == 4) ? cur : lay;
-  k_scan_counts<<<1, 1024, 0, st>>>(s.count[cntlay], s.ncells, s.tmp_start);
+  launch_scan(s.count[cntlay], s.ncells, s.tmp_start, st);
   const int blocks = (s.ncells + WPB - 1) / WPB;
   k_export<T><<<blocks, WPB * 32, 0, st>>>(s.buf[cur], s.start[lay], s.count[cntlay], s.tmp_start, s.ncells, x, y,
                                           vx, vy, vz, ir, cell);
@@ -1862,9 +2166,13 @@ void Ops<T>::import_particles(const Params<T>& p, State<T>& s, int& cur, int& la
   const double* yy = (p.dim == 2) ? y : x;  // y is not read in 1D; pass any valid pointer
   s.nparticles = (int)n;
   if (det) {
-    // stable sort of the input into the other buffer: the compact layout
-    k_sort_stable<double, T><<<1, 1024, 0, st>>>(x, yy, vx, vy, vz, ir, s.buf[other], s.key, (int)n, p.ncells,
-                                                 s.start[olay], s.count[olay], s.tmp2, s.dest, s.cellof);
+    if constexpr (sizeof(T) == 8) {
+      // sorted by cell into the other buffer, in the given order within a cell
+      cudaMemsetAsync(s.count[olay], 0, sizeof(int32_t) * (size_t)s.ncells, st);
+      if (n > 0) k_arrivals<<<grid_for(n, 256), 256, 0, st>>>(s.key, (int)n, s.count[olay], s.dest);
+      det_cells<T>(p, s, (int)n, x, yy, vx, vy, vz, ir, other, olay, 0u, 0, false, st);
+      s.count_clear = false;
+    }
     cur = other;
     lay = olay;
     if (p.mesh == 1) {
@@ -1906,7 +2214,7 @@ void Ops<T>::dig_counts(State<T>& s, int ncells, int lay, const double* target, 
   // caps go to tmp_start (ncells), then scanned into the other layout's start
   k_dig_counts<<<grid_for(ncells, 256), 256, 0, st>>>(s.cases.cp, s.cases.cell_case, s.cases.cell0, ncells, target,
                                                       iter, det, s.slack, s.nt, s.tmp_start, s.flags);
-  k_scan_caps<<<1, 1024, 0, st>>>(s.tmp_start, ncells, (long long)s.capacity, s.start[lay ^ 1], s.flags);
+  launch_scan(s.tmp_start, ncells, s.start[lay ^ 1], st, s.flags + 1, s.flags, (long long)s.capacity);
 }
 
 template <typename T>
@@ -1927,14 +2235,15 @@ void Ops<T>::dig_apply(const CellParams& cp0, State<T>& s, int ncells, int& cur,
                                                     s.buf[other], s.start[lay], s.count[cin], s.start[olay],
                                                     s.count[cout], s.nt, target, iter, s.scratch_i,
                                                     det ? s.cellof : nullptr, s.tile);
-  if (!det) k_zero_i32<<<grid_for(ncells, 256), 256, 0, st>>>(s.count[cur], ncells);
+  if (det) s.count_clear = false;
+  else k_zero_i32<<<grid_for(ncells, 256), 256, 0, st>>>(s.count[cur], ncells);
   cur = other;
   lay = olay;
 }
 
 template <typename T>
 void Ops<T>::total_count(State<T>& s, const int32_t* cnt, int ncells, cudaStream_t st) {
-  k_scan_counts<<<1, 1024, 0, st>>>(cnt, ncells, s.tmp_start);
+  launch_scan(cnt, ncells, s.tmp_start, st);
 }
 
 template <typename T>
@@ -1947,8 +2256,13 @@ void Ops<T>::configure(int tile) {
   tile = TILE_MAX_OF<T>;
   const int sm = (int)tile_smem<T>(tile);
   const int smd = WPB * tile * 2 * (int)sizeof(int32_t);
-  cudaFuncSetAttribute(k_collide_sample<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-  cudaFuncSetAttribute(k_collide_sample<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  if constexpr (sizeof(T) == 8) {
+    cudaFuncSetAttribute(k_det_cells<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(k_det_cells<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  } else {
+    cudaFuncSetAttribute(k_collide_sample<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(k_collide_sample<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+  }
   cudaFuncSetAttribute(k_dig_apply<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smd);
   cudaFuncSetAttribute(k_dig_apply<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smd);
   if constexpr (sizeof(T) == 4) {
