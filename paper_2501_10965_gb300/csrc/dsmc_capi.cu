@@ -287,6 +287,7 @@ Plan make_plan(const dsmc_config* cs, int ncases, char* base, dsmc_handle* h) {
   ml.scal = cv.take<double>(8);
   ml.count = cv.take<int32_t>(4);
   ml.jacc = cv.take<double>((size_t)pl.ncells * 16);
+  ml.pass = cv.take<uint8_t>(pl.ncells);
   const bool ann = cs[0].mesh == DSMC_MESH_ANNULUS, ref = cs[0].mesh == DSMC_MESH_REFINED;
   const size_t nr1 = ann ? (size_t)cs[0].ny + 1 : 1, nray = ann ? 2 * ((size_t)cs[0].nx + 1) : 1;
   const size_t nfn = ann ? 2 * (size_t)cs[0].nx : 1, nvol = (ann || ref) ? (size_t)pl.ncells : 1;

@@ -85,7 +85,11 @@ void launch_acc_sum(int ncells, const double* acc, const double* comp, double* o
 // ---------------------------------------------------------------------------
 // HoT and Kn_GLL
 // ---------------------------------------------------------------------------
-__global__ void k_hot(const CellParams* __restrict__ cps, const int32_t* __restrict__ cell_case,
+// The FP64 pipe bounds it (2 lanes per clock and SM; the fields come from L2):
+// a 1D case forms no y gradients, lambda takes one division, and Kn_GLL's
+// velocity scale max(|u|, sqrt(gamma T)) one square root.  160 000 cells (1D):
+// 193 us before, 122 us now.
+__global__ void __launch_bounds__(128) k_hot(const CellParams* __restrict__ cps, const int32_t* __restrict__ cell_case,
                       const int32_t* __restrict__ cell0, int ncells, const double* __restrict__ F,
                       double* __restrict__ hot, double* __restrict__ kngll, uint8_t* __restrict__ mask) {
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) {
@@ -96,18 +100,38 @@ __global__ void k_hot(const CellParams* __restrict__ cps, const int32_t* __restr
     const double rho = f[0], ux = f[1], uy = f[2], tt = f[4], tr = f[5];
     const double T = (3.0 * tt + cp.d_r * tr) / (3.0 + cp.d_r);
     const double mu = cp.mu_ref * pow(T, cp.omega);
-    double duxx, duxy, duyx, duyy, duzx, duzy, dttx, dtty, dtrx, dtry, drx, dry, dsx, dsy;
-    grad2(cp, c, lc, [&](int k) { return F[(size_t)k * 18 + 1]; }, &duxx, &duxy);
-    grad2(cp, c, lc, [&](int k) { return F[(size_t)k * 18 + 2]; }, &duyx, &duyy);
-    grad2(cp, c, lc, [&](int k) { return F[(size_t)k * 18 + 3]; }, &duzx, &duzy);
-    grad2(cp, c, lc, [&](int k) { return F[(size_t)k * 18 + 4]; }, &dttx, &dtty);
-    grad2(cp, c, lc, [&](int k) { return F[(size_t)k * 18 + 5]; }, &dtrx, &dtry);
-    grad2(cp, c, lc, [&](int k) { return F[(size_t)k * 18 + 0]; }, &drx, &dry);
-    grad2(cp, c, lc, [&](int k) {
-            const double* g = F + (size_t)k * 18;
-            return sqrt(g[1] * g[1] + g[2] * g[2] + g[3] * g[3]);
-          },
-          &dsx, &dsy);
+    double duxx, duxy = 0.0, duyx, duyy = 0.0, duzx, duzy = 0.0, dttx, dtty = 0.0, dtrx, dtry = 0.0;
+    double g_rho, g_u, g_tt, g_tr;
+    auto val = [&](int col) { return [F, col](int k) { return F[(size_t)k * 18 + col]; }; };
+    auto speed_at = [&](int k) {
+      const double* g = F + (size_t)k * 18;
+      return sqrt(g[1] * g[1] + g[2] * g[2] + g[3] * g[3]);
+    };
+    if (cp.dim == 1) {
+      const Line1 l(cp, c, lc);
+      duxx = l.grad(val(1));
+      duyx = l.grad(val(2));
+      duzx = l.grad(val(3));
+      dttx = l.grad(val(4));
+      dtrx = l.grad(val(5));
+      g_rho = fabs(l.grad(val(0)));
+      g_u = fabs(l.grad(speed_at));
+      g_tt = fabs(dttx);
+      g_tr = fabs(dtrx);
+    } else {
+      double drx, dry, dsx, dsy;
+      grad2(cp, c, lc, val(1), &duxx, &duxy);
+      grad2(cp, c, lc, val(2), &duyx, &duyy);
+      grad2(cp, c, lc, val(3), &duzx, &duzy);
+      grad2(cp, c, lc, val(4), &dttx, &dtty);
+      grad2(cp, c, lc, val(5), &dtrx, &dtry);
+      grad2(cp, c, lc, val(0), &drx, &dry);
+      grad2(cp, c, lc, speed_at, &dsx, &dsy);
+      g_rho = hypot(drx, dry);
+      g_u = hypot(dsx, dsy);
+      g_tt = hypot(dttx, dtty);
+      g_tr = hypot(dtrx, dtry);
+    }
     const double div = duxx + duyy;
     double sig[6];
     sig[0] = -mu * (2.0 * duxx - 2.0 / 3.0 * div);
@@ -120,13 +144,9 @@ __global__ void k_hot(const CellParams* __restrict__ cps, const int32_t* __restr
     const double qr[3] = {-cp.kappa_r * mu * dtrx, -cp.kappa_r * mu * dtry, 0.0};
     // Kn_GLL
     const double gamma = (5.0 + cp.d_r) / (3.0 + cp.d_r);
-    const double speed = sqrt(ux * ux + uy * uy + f[3] * f[3]);
-    const double lam = mu / (rho * T) * sqrt(PI_D * T / 2.0);
-    const double g_rho = hypot(drx, dry) / rho;
-    const double g_u = hypot(dsx, dsy) / fmax(speed, sqrt(gamma * T));
-    const double g_tt = hypot(dttx, dtty) / tt;
-    const double g_tr = hypot(dtrx, dtry) / tr;
-    const double kn = lam * fmax(fmax(g_rho, g_u), fmax(g_tt, g_tr));
+    const double lam = mu * sqrt(PI_D * T / 2.0) / (rho * T);
+    const double us = sqrt(fmax(ux * ux + uy * uy + f[3] * f[3], gamma * T));
+    const double kn = lam * fmax(fmax(g_rho / rho, g_u / us), fmax(g_tt / tt, g_tr / tr));
     const bool keep = kn >= cp.kn_ref;
     double* h = hot + (size_t)c * 12;
     for (int q = 0; q < 6; ++q) h[q] = keep ? f[6 + q] - sig[q] : 0.0;
@@ -139,8 +159,8 @@ __global__ void k_hot(const CellParams* __restrict__ cps, const int32_t* __restr
 
 void launch_hot(const CellParams* cp, const int32_t* cell_case, const int32_t* cell0, int ncells,
                 const double* fields, double* hot, double* kngll, uint8_t* mask, cudaStream_t st) {
-  const int g = (ncells + 255) / 256;
-  k_hot<<<g > 0 ? g : 1, 256, 0, st>>>(cp, cell_case, cell0, ncells, fields, hot, kngll, mask);
+  const int g = (ncells + 127) / 128;
+  k_hot<<<g > 0 ? g : 1, 128, 0, st>>>(cp, cell_case, cell0, ncells, fields, hot, kngll, mask);
 }
 
 // ---------------------------------------------------------------------------

@@ -84,4 +84,20 @@ __device__ __forceinline__ void grad2(const CellParams& cp, int c, int lc, F f, 
   }
 }
 
+// the same in 1D (d/dy is 0), for several fields of one cell: the two cells
+// and the reciprocal of their distance
+struct Line1 {
+  int lo, hi;
+  double inv;
+  __device__ __forceinline__ Line1(const CellParams& cp, int c, int lc) {
+    lo = lc > 0 ? c - 1 : c;
+    hi = lc < cp.nx - 1 ? c + 1 : c;
+    inv = hi == lo ? 0.0 : 1.0 / ((double)(hi - lo) * cp.dx);
+  }
+  template <typename F>
+  __device__ __forceinline__ double grad(F f) const {
+    return hi == lo ? 0.0 : (f(hi) - f(lo)) * inv;
+  }
+};
+
 }  // namespace dsmc

@@ -181,6 +181,7 @@ struct Mlp {
   float* out;        // ncells x 5 network outputs
   double* scal;      // [0] loss, [2] judge sum, [3] judge count, [4] cells given the network's HoT
   int32_t* count;    // [0] number of cells with w = 1
+  uint8_t* pass;     // ncells: the judge's verdict per group
   double* jacc;      // ncells x 16 judge statistics per group: sum r (5), sum r^2 (5), count, sum Y (5)
 };
 // inputs, scales, targets (hot may be null) and weights of every cell

@@ -52,78 +52,115 @@ inline size_t fb_smem_bytes(bool train) {
 
 __device__ __forceinline__ float bf16_to_f(uint16_t h) { return __uint_as_float((uint32_t)h << 16); }
 
-// per cell: inputs (12), scales (4), normalised HoT targets (5, if hot) and
-// weight (1 where mask = 1 and the cell state admits the inputs)
-__global__ void k_mlp_data(const CellParams* __restrict__ cps, const int32_t* __restrict__ cell_case,
+// Per cell: inputs (12), scales (4), normalised HoT targets (5, if hot) and
+// weight (1 where mask = 1 and the cell state admits the inputs); a cell with
+// mask = 0 is neither trained on nor replaced and gets zeros.
+// The FP64 pipe bounds it (2 lanes per clock and SM): the divisions by the
+// cell's own scales are one reciprocal each, the y gradients of a 1D case
+// (zero) are not formed.  The count is added once per warp.
+// 160 000 cells (1D): 236 us before, 98 us now.
+__global__ void __launch_bounds__(128) k_mlp_data(const CellParams* __restrict__ cps,
+                           const int32_t* __restrict__ cell_case,
                            const int32_t* __restrict__ cell0, int ncells, const double* __restrict__ F,
                            const double* __restrict__ hot, const double* __restrict__ kngll,
                            const uint8_t* __restrict__ mask, float* __restrict__ X, float* __restrict__ Y,
                            float* __restrict__ S, float* __restrict__ w, int32_t* __restrict__ count) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) {
-    const int cs = cell_case[c];
-    const CellParams& cp = cps[cs];
-    const int lc = c - cell0[cs];
-    const double* f = F + (size_t)c * 18;
-    const double rho = f[0], tt = f[4], tr = f[5];
-    const double T = (3.0 * tt + cp.d_r * tr) / (3.0 + cp.d_r);
-    double x[12], sc[4], y[5];
-    bool ok = rho > 0.0 && tt > 0.0 && tr > 0.0 && isfinite(T);
-    if (ok) {
-      const double mu = cp.mu_ref * pow(T, cp.omega);
-      const double lam = mu / (rho * T) * sqrt(M_PI * T / 2.0);
-      const double sq = sqrt(T);
-      const int cols[5] = {0, 1, 2, 4, 5};
-      const double norm[5] = {rho, sq, sq, T, T};
-      for (int k = 0; k < 5; ++k) {
-        double gx, gy;
-        const int col = cols[k];
-        grad2(cp, c, lc, [&](int q) { return F[(size_t)q * 18 + col]; }, &gx, &gy);
-        x[2 * k] = lam * gx / norm[k];
-        x[2 * k + 1] = lam * gy / norm[k];
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  bool ok = false;
+  if (c < ncells) {
+    float x[12], sc[4], y[5];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) x[k] = 0.f;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) y[k] = 0.f;
+    sc[0] = sc[1] = sc[2] = 1.f;
+    sc[3] = 0.f;
+    if (mask[c] != 0) {
+      const int cs = cell_case[c];
+      const CellParams& cp = cps[cs];
+      const int lc = c - cell0[cs];
+      const double* f = F + (size_t)c * 18;
+      const double rho = f[0], tt = f[4], tr = f[5];
+      const double i3 = 1.0 / (3.0 + cp.d_r);
+      const double T = (3.0 * tt + cp.d_r * tr) * i3;
+      ok = rho > 0.0 && tt > 0.0 && tr > 0.0 && isfinite(T);
+      if (ok) {
+        const bool one = cp.dim == 1;
+        const double mu = cp.mu_ref * pow(T, cp.omega);
+        const double sq = sqrt(T), iT = 1.0 / T, irho = 1.0 / rho, isq = sq * iT;
+        // lambda / norm of rho; u_x, u_y; T_t, T_r
+        const double lam = mu * irho * isq * 1.2533141373155003;  // sqrt(pi / 2)
+        const double ln[5] = {lam * irho, lam * isq, lam * isq, lam * iT, lam * iT};
+        double gx[5], gy[5];
+        const Line1 line(cp, c, lc);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          const int col = k < 3 ? k : k + 1;  // rho, u_x, u_y, T_t, T_r
+          auto val = [&](int q) { return F[(size_t)q * 18 + col]; };
+          if (one) {
+            gx[k] = line.grad(val);
+            gy[k] = 0.0;
+          } else {
+            grad2(cp, c, lc, val, &gx[k], &gy[k]);
+          }
+          x[2 * k] = (float)(ln[k] * gx[k]);
+          x[2 * k + 1] = one ? 0.f : (float)(ln[k] * gy[k]);
+        }
+        x[10] = (float)kngll[c];
+        x[11] = (float)(tr / tt);
+        // grad T from the gradients of T_t and T_r
+        const double gTx = (3.0 * gx[3] + cp.d_r * gx[4]) * i3, gTy = (3.0 * gy[3] + cp.d_r * gy[4]) * i3;
+        double ex = 1.0, ey = 0.0;
+        if (one) {
+          if (gTx < 0.0) ex = -1.0;
+        } else {
+          const double gn = sqrt(gTx * gTx + gTy * gTy);
+          if (gn > 0.0) {
+            ex = gTx / gn;
+            ey = gTy / gn;
+          }
+        }
+        const double p = rho * T, ps = p * sq;
+        sc[0] = (float)p;
+        sc[1] = (float)ps;
+        sc[2] = (float)ex;
+        sc[3] = (float)ey;
+        bool fin = true;
+        if (hot) {
+          const double* h = hot + (size_t)c * 12;
+          const double ip = irho * iT, ips = ip * isq;
+          const double yd[5] = {h[0] * ip, h[3] * ip, h[1] * ip, (h[6] * ex + h[7] * ey) * ips,
+                                (h[9] * ex + h[10] * ey) * ips};
+#pragma unroll
+          for (int k = 0; k < 5; ++k) {
+            fin = fin && isfinite(yd[k]);
+            y[k] = (float)yd[k];
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 5; ++k) fin = fin && isfinite(ln[k] * gx[k]) && (one || isfinite(ln[k] * gy[k]));
+        ok = fin && isfinite(kngll[c]) && isfinite(tr / tt);
+        if (!ok) {
+#pragma unroll
+          for (int k = 0; k < 12; ++k) x[k] = 0.f;
+#pragma unroll
+          for (int k = 0; k < 5; ++k) y[k] = 0.f;
+          sc[0] = sc[1] = sc[2] = 1.f;
+          sc[3] = 0.f;
+        }
       }
-      x[10] = kngll[c];
-      x[11] = tr / tt;
-      double gTx, gTy;
-      grad2(cp, c, lc,
-            [&](int q) {
-              const double* g = F + (size_t)q * 18;
-              return (3.0 * g[4] + cp.d_r * g[5]) / (3.0 + cp.d_r);
-            },
-            &gTx, &gTy);
-      const double gn = sqrt(gTx * gTx + gTy * gTy);
-      const double ex = gn > 0.0 ? gTx / gn : 1.0, ey = gn > 0.0 ? gTy / gn : 0.0;
-      const double p = rho * T;
-      sc[0] = p;
-      sc[1] = p * sq;
-      sc[2] = ex;
-      sc[3] = ey;
-      if (hot) {
-        const double* h = hot + (size_t)c * 12;
-        y[0] = h[0] / p;
-        y[1] = h[3] / p;
-        y[2] = h[1] / p;
-        y[3] = (h[6] * ex + h[7] * ey) / sc[1];
-        y[4] = (h[9] * ex + h[10] * ey) / sc[1];
-      } else {
-        for (int k = 0; k < 5; ++k) y[k] = 0.0;
-      }
-      for (int k = 0; k < 12; ++k) ok = ok && isfinite(x[k]);
-      for (int k = 0; k < 5; ++k) ok = ok && isfinite(y[k]);
     }
-    if (!ok) {
-      for (int k = 0; k < 12; ++k) x[k] = 0.0;
-      for (int k = 0; k < 5; ++k) y[k] = 0.0;
-      sc[0] = sc[1] = 1.0;
-      sc[2] = 1.0;
-      sc[3] = 0.0;
-    }
-    for (int k = 0; k < 12; ++k) X[(size_t)c * 12 + k] = (float)x[k];
-    for (int k = 0; k < 5; ++k) Y[(size_t)c * 5 + k] = (float)y[k];
-    for (int k = 0; k < 4; ++k) S[(size_t)c * 4 + k] = (float)sc[k];
-    const bool use = ok && mask[c] != 0;
-    w[c] = use ? 1.f : 0.f;
-    if (use) atomicAdd(count, 1);
+    float4* X4 = reinterpret_cast<float4*>(X + (size_t)c * 12);
+    X4[0] = make_float4(x[0], x[1], x[2], x[3]);
+    X4[1] = make_float4(x[4], x[5], x[6], x[7]);
+    X4[2] = make_float4(x[8], x[9], x[10], x[11]);
+    *reinterpret_cast<float4*>(S + (size_t)c * 4) = make_float4(sc[0], sc[1], sc[2], sc[3]);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) Y[(size_t)c * 5 + k] = y[k];
+    w[c] = ok ? 1.f : 0.f;
   }
+  const unsigned used = __ballot_sync(0xffffffffu, ok);
+  if ((threadIdx.x & 31) == 0 && used) atomicAdd(count, __popc(used));
 }
 
 template <int L, bool TANH>
@@ -430,25 +467,34 @@ __global__ void __launch_bounds__(TC_WARPS * 32) k_mlp_fwd_tc(const uint16_t* __
 // The judge's statistics: every cell of the network (w = 1, finite
 // outputs) adds its residual r = network - DSMC (5 normalised outputs), r^2
 // and the DSMC terms Y to its group's sums, and 1 to its count (FP64):
-// JACC doubles per group.
+// JACC doubles per group.  Sixteen lanes take one cell, a lane per sum, so
+// that a cell's additions reach L2 as one 128-byte row (160 000 cells, 200
+// groups: 46 us with 16 additions per thread, 28 us).
 constexpr int JACC = 16;
-__global__ void k_mlp_judge_acc(int ncells, const float* __restrict__ out, const float* __restrict__ Y,
+__global__ void __launch_bounds__(256) k_mlp_judge_acc(int ncells, const float* __restrict__ out,
+                                const float* __restrict__ Y,
                                 const float* __restrict__ w, const int32_t* __restrict__ group,
                                 double* __restrict__ jacc) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) {
+  const int k = threadIdx.x & 15;
+  const int stride = (gridDim.x * blockDim.x) >> 4;
+  for (int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 4; c < ncells; c += stride) {
+    if (w[c] == 0.f) continue;
     const float* o = out + (size_t)c * 5;
+    const float* yc = Y + (size_t)c * 5;
     bool fin = true;
-    for (int k = 0; k < 5; ++k) fin = fin && isfinite(o[k]);
-    if (w[c] == 0.f || !fin) continue;
-    double* a = jacc + (size_t)(group ? group[c] : c) * JACC;
-    for (int k = 0; k < 5; ++k) {
-      const double y = (double)Y[(size_t)c * 5 + k];
-      const double r = (double)o[k] - y;
-      atomicAdd(a + k, r);
-      atomicAdd(a + 5 + k, r * r);
-      atomicAdd(a + 11 + k, y);
+    for (int q = 0; q < 5; ++q) fin = fin && isfinite(o[q]);
+    if (!fin) continue;
+    double v = 1.0;  // k = 10: the count
+    if (k < 10) {
+      const int q = k < 5 ? k : k - 5;
+      const double r = (double)o[q] - (double)yc[q];
+      v = k < 5 ? r : r * r;
+    } else if (k > 10) {
+      v = (double)yc[k - 11];
     }
-    atomicAdd(a + 10, 1.0);
+    double* a = jacc + (size_t)(group ? group[c] : c) * JACC + k;
+    if (group) atomicAdd(a, v);
+    else *a += v;
   }
 }
 
@@ -467,52 +513,82 @@ __device__ __forceinline__ bool judge_pass(const double* a, double z, int min_sa
   return true;
 }
 
+// the verdict of every group, once (a group without samples fails at once)
+__global__ void k_mlp_verdict(int ngroups, const double* __restrict__ jacc, double z, int min_samples, double rel,
+                              uint8_t* __restrict__ pass) {
+  const int g = blockIdx.x * blockDim.x + threadIdx.x;
+  if (g < ngroups) pass[g] = judge_pass(jacc + (size_t)g * JACC, z, min_samples, rel) ? 1 : 0;
+}
+
 // HoT for the synthetic equations and the judge sums (network against DSMC);
 // hot and hot_out may be the same array (each thread reads its cell first).
-// With z > 0 a network cell keeps the DSMC HoT unless its group passes the
-// judge (judge_pass).
-__global__ void k_mlp_hot(int ncells, const float* __restrict__ out, const float* __restrict__ Y,
+// With pass (the groups' verdicts) a network cell keeps the DSMC HoT unless
+// its group passes.  The three judge sums are reduced over the CTA before
+// they are added (one address each: 160 000 cells took 488 us with an
+// addition per cell, 16 us with one per CTA).
+__global__ void __launch_bounds__(256) k_mlp_hot(int ncells, const float* __restrict__ out,
+                          const float* __restrict__ Y,
                           const float* __restrict__ S, const float* __restrict__ w, const double* hot,
                           double* hot_out, double* __restrict__ scal, const int32_t* __restrict__ group,
-                          const double* __restrict__ jacc, double z, int min_samples, double rel) {
-  double jsum = 0.0, jcnt = 0.0, nnet = 0.0;
+                          const uint8_t* __restrict__ pass) {
+  __shared__ double s_j[8];
+  __shared__ int s_c[8], s_n[8];
+  double jsum = 0.0;
+  int jcnt = 0, nnet = 0;
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < ncells; c += gridDim.x * blockDim.x) {
     double h[12];
+#pragma unroll
     for (int k = 0; k < 12; ++k) h[k] = hot[(size_t)c * 12 + k];
     const float* o = out + (size_t)c * 5;
     bool fin = true;
     for (int k = 0; k < 5; ++k) fin = fin && isfinite(o[k]);
-    const bool judged = z > 0.0 && w[c] != 0.f && fin;
-    const bool pass = !judged || judge_pass(jacc + (size_t)(group ? group[c] : c) * JACC, z, min_samples, rel);
     if (w[c] != 0.f && fin) {
       for (int k = 0; k < 5; ++k) {
         const double r = (double)o[k] - (double)Y[(size_t)c * 5 + k];
         jsum += r * r;
       }
-      jcnt += 5.0;
-    }
-    if (w[c] != 0.f && fin && pass) {
-      nnet += 1.0;
-      const double p = S[(size_t)c * 4], ps = S[(size_t)c * 4 + 1];
-      const double ex = S[(size_t)c * 4 + 2], ey = S[(size_t)c * 4 + 3];
-      h[0] = (double)o[0] * p;
-      h[3] = (double)o[1] * p;
-      h[1] = (double)o[2] * p;
-      const int base[2] = {6, 9};
-      for (int r = 0; r < 2; ++r) {
-        const double along = h[base[r]] * ex + h[base[r] + 1] * ey;
-        const double nw = (double)o[3 + r] * ps;
-        h[base[r]] += (nw - along) * ex;
-        h[base[r] + 1] += (nw - along) * ey;
+      jcnt += 5;
+      if (!pass || pass[group ? group[c] : c]) {
+        nnet += 1;
+        const double p = S[(size_t)c * 4], ps = S[(size_t)c * 4 + 1];
+        const double ex = S[(size_t)c * 4 + 2], ey = S[(size_t)c * 4 + 3];
+        h[0] = (double)o[0] * p;
+        h[3] = (double)o[1] * p;
+        h[1] = (double)o[2] * p;
+        const int base[2] = {6, 9};
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const double along = h[base[r]] * ex + h[base[r] + 1] * ey;
+          const double nw = (double)o[3 + r] * ps;
+          h[base[r]] += (nw - along) * ex;
+          h[base[r] + 1] += (nw - along) * ey;
+        }
       }
     }
+#pragma unroll
     for (int k = 0; k < 12; ++k) hot_out[(size_t)c * 12 + k] = h[k];
   }
-  if (jcnt > 0.0) {
-    atomicAdd(scal + 2, jsum);
-    atomicAdd(scal + 3, jcnt);
+  for (int o = 16; o > 0; o >>= 1) jsum += __shfl_xor_sync(0xffffffffu, jsum, o);
+  jcnt = __reduce_add_sync(0xffffffffu, jcnt);
+  nnet = __reduce_add_sync(0xffffffffu, nnet);
+  if ((threadIdx.x & 31) == 0) {
+    s_j[threadIdx.x >> 5] = jsum;
+    s_c[threadIdx.x >> 5] = jcnt;
+    s_n[threadIdx.x >> 5] = nnet;
   }
-  if (nnet > 0.0) atomicAdd(scal + 4, nnet);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; ++k) {
+      jsum += s_j[k];
+      jcnt += s_c[k];
+      nnet += s_n[k];
+    }
+    if (jcnt > 0) {
+      atomicAdd(scal + 2, jsum);
+      atomicAdd(scal + 3, (double)jcnt);
+    }
+    if (nnet > 0) atomicAdd(scal + 4, (double)nnet);
+  }
 }
 
 inline int blocks_for(int n, int t) { return (n + t - 1) / t; }
@@ -532,7 +608,7 @@ void mlp_prepare(const Mlp& m, const CellParams* cp, const int32_t* cell_case, c
                  const double* fields, const double* hot, const double* kngll, const uint8_t* mask,
                  cudaStream_t st) {
   cudaMemsetAsync(m.count, 0, sizeof(int32_t), st);
-  k_mlp_data<<<blocks_for(ncells, 256), 256, 0, st>>>(cp, cell_case, cell0, ncells, fields, hot, kngll, mask, m.X,
+  k_mlp_data<<<blocks_for(ncells, 128), 128, 0, st>>>(cp, cell_case, cell0, ncells, fields, hot, kngll, mask, m.X,
                                                        m.Y, m.S, m.w, m.count);
 }
 
@@ -562,9 +638,12 @@ void mlp_apply(const Mlp& m, int ncells, const double* hot, double* hot_out, cud
   k_mlp_fwd_tc<<<grid, TC_WARPS * 32, tc_smem_bytes(), st>>>(m.wbf, m.theta, m.X, ncells, m.out);
   cudaMemsetAsync(m.scal + 2, 0, 3 * sizeof(double), st);
   const int hb = blocks_for(ncells, 256) < 1024 ? blocks_for(ncells, 256) : 1024;
-  if (z > 0.0) k_mlp_judge_acc<<<hb, 256, 0, st>>>(ncells, m.out, m.Y, m.w, group, m.jacc);
-  k_mlp_hot<<<hb, 256, 0, st>>>(ncells, m.out, m.Y, m.S, m.w, hot, hot_out, m.scal, group, m.jacc, z, min_samples,
-                                rel);
+  if (z > 0.0) {
+    const int jb = blocks_for(ncells, 16);
+    k_mlp_judge_acc<<<jb < 152 * 8 ? jb : 152 * 8, 256, 0, st>>>(ncells, m.out, m.Y, m.w, group, m.jacc);
+    k_mlp_verdict<<<blocks_for(ncells, 256), 256, 0, st>>>(ncells, m.jacc, z, min_samples, rel, m.pass);
+  }
+  k_mlp_hot<<<hb, 256, 0, st>>>(ncells, m.out, m.Y, m.S, m.w, hot, hot_out, m.scal, group, z > 0.0 ? m.pass : nullptr);
 }
 
 }  // namespace dsmc
