@@ -1490,6 +1490,16 @@ __global__ void k_rebin_ovf(const Ovf ov, int ovf_cap, PBuf<float> out, const in
 // ---------------------------------------------------------------------------
 // export / import
 // ---------------------------------------------------------------------------
+// float -> double by integer operations where the value is normal (the
+// conversion instruction runs on the FP64 pipe at 2 lanes per clock and SM)
+__device__ __forceinline__ double f2d(float v) {
+  const uint32_t u = __float_as_uint(v), e = u & 0x7f800000u;
+  if (e == 0u || e == 0x7f800000u) return (double)v;
+  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ double to_double(float v) { return f2d(v); }
+__device__ __forceinline__ double to_double(double v) { return v; }
+
 template <typename T>
 __global__ void __launch_bounds__(WPB * 32) k_export(PBuf<T> b, const int32_t* __restrict__ start,
                                                      const int32_t* __restrict__ cnt,
@@ -1501,12 +1511,12 @@ __global__ void __launch_bounds__(WPB * 32) k_export(PBuf<T> b, const int32_t* _
   if (cell >= ncells) return;
   const int si = start[cell], so = ostart[cell], n = cnt[cell];
   for (int q = lane; q < n; q += 32) {
-    x[so + q] = (double)b.x[si + q];
-    y[so + q] = (double)b.y[si + q];
-    vx[so + q] = (double)b.vx[si + q];
-    vy[so + q] = (double)b.vy[si + q];
-    vz[so + q] = (double)b.vz[si + q];
-    ir[so + q] = (double)b.ir[si + q];
+    x[so + q] = to_double(b.x[si + q]);
+    y[so + q] = to_double(b.y[si + q]);
+    vx[so + q] = to_double(b.vx[si + q]);
+    vy[so + q] = to_double(b.vy[si + q]);
+    vz[so + q] = to_double(b.vz[si + q]);
+    ir[so + q] = to_double(b.ir[si + q]);
     cell_out[so + q] = cell;
   }
 }
@@ -1628,31 +1638,48 @@ static __global__ void k_dig_counts(const CellParams* __restrict__ cps, const in
   }
 }
 
+// a new particle's position: uniform in the cell
+template <typename T>
+__device__ __forceinline__ void dig_position(const CellParams& cp, Stream<double>& sp, int ix, int iy, T* x, T* y) {
+  if (cp.mesh == 1) {
+    // annulus: uniform in the sector (r^2 and the angle uniform)
+    const double r = sqrt(cp.r2t[iy] + sp.u(0) * (cp.r2t[iy + 1] - cp.r2t[iy]));
+    const double th = 2.0 * PI_D * ((double)ix + sp.u(1)) / (double)cp.nx;
+    *x = (T)(r * cos(th));
+    *y = (T)(r * sin(th));
+  } else if (cp.mesh == 2) {
+    // wall-refined box: uniform between the cell's edges
+    *x = (T)(cp.xe[ix] + sp.u(0) * (cp.xe[ix + 1] - cp.xe[ix]));
+    *y = (T)(cp.ye[iy] + sp.u(1) * (cp.ye[iy + 1] - cp.ye[iy]));
+  } else {
+    *x = (T)(((double)ix + sp.u(0)) * cp.dx);
+    *y = (T)((cp.dim == 2) ? ((double)iy + sp.u(1)) * cp.dy : 0.0);
+  }
+}
+
+// removal q of n: partial Fisher-Yates draw r_q = q + floor(u_q (n - q))
+__device__ __forceinline__ int dig_removal(const CellParams& cp, int q, int n, int lcell, uint32_t iter) {
+  Stream<double> st(TAG_DIG_SEL, (uint32_t)q, (uint32_t)lcell, iter, cp.k0, cp.k1);
+  const int r = q + (int)(st.u(0) * (double)(n - q));
+  return r > n - 1 ? n - 1 : r;
+}
+
+// source of added particle q in a cell of n
+__device__ __forceinline__ int dig_source(const CellParams& cp, int q, int n, int lcell, uint32_t iter) {
+  Stream<double> ss(TAG_DIG_SEL, (uint32_t)q, (uint32_t)lcell, iter, cp.k0, cp.k1);
+  const int r = (int)(ss.u(0) * (double)n);
+  return r > n - 1 ? n - 1 : r;
+}
+
+// Steps ii-iv for one cell of any size and precision by its warp, through the
+// output arrays.  idx: n ints; rm: n ints of shared memory, or null when idx
+// lies in global memory.
 template <typename T, int DIM>
-__global__ void __launch_bounds__(WPB * 32) k_dig_apply(const CellParams* __restrict__ cps,
-                                                        const int32_t* __restrict__ cell_case,
-                                                        const int32_t* __restrict__ cell0, int ncells,
-                                                        PBuf<T> in, PBuf<T> out,
-                                                        const int32_t* __restrict__ start_in,
-                                                        const int32_t* __restrict__ cnt_in,
-                                                        const int32_t* __restrict__ start_out,
-                                                        int32_t* __restrict__ cnt_out,
-                                                        const int32_t* __restrict__ nt,
-                                                        const double* __restrict__ target, uint32_t iter,
-                                                        int32_t* __restrict__ idx_g,
-                                                        int32_t* __restrict__ cellof_out, int tile) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int cell = blockIdx.x * WPB + warp;
-  if (cell >= ncells) return;
-  const int cs = cell_case[cell];
-  const CellParams& cp = cps[cs];
-  const int lcell = cell - cell0[cs];
-  const int s0 = start_in[cell], n = cnt_in[cell], d0 = start_out[cell], ntg = nt[cell];
-  const double* t = target + (size_t)cell * 6;
+__device__ void dig_cell(const CellParams& cp, int cell, int lcell, const PBuf<T>& in, const PBuf<T>& out, int s0,
+                         int n, int d0, int ntg, const double* __restrict__ t, uint32_t iter, int32_t* idx,
+                         int32_t* rm, int32_t* __restrict__ cellof_out) {
+  const int lane = threadIdx.x & 31;
   const int ix = lcell % cp.nx, iy = lcell / cp.nx;
-  int32_t* idx = (n <= tile) ? reinterpret_cast<int32_t*>(smem) + (size_t)warp * tile * 2 : idx_g + s0;
-  int32_t* rm = (n <= tile) ? reinterpret_cast<int32_t*>(smem) + (size_t)warp * tile * 2 + tile : nullptr;
   // step ii
   if (ntg <= n) {
     const int k = n - ntg;
@@ -1665,11 +1692,7 @@ __global__ void __launch_bounds__(WPB * 32) k_dig_apply(const CellParams* __rest
       for (int qb = 0; qb < k; qb += 32) {
         const int q = qb + lane;
         int r = 0;
-        if (q < k) {
-          Stream<double> st(TAG_DIG_SEL, (uint32_t)q, (uint32_t)lcell, iter, cp.k0, cp.k1);
-          r = q + (int)(st.u(0) * (double)(n - q));
-          if (r > n - 1) r = n - 1;
-        }
+        if (q < k) r = dig_removal(cp, q, n, lcell, iter);
         const int m = min(32, k - qb);
         for (int j = 0; j < m; ++j) {
           const int rj = __shfl_sync(FULL, r, j);
@@ -1731,24 +1754,12 @@ __global__ void __launch_bounds__(WPB * 32) k_dig_apply(const CellParams* __rest
     for (int q = lane; q < ntg - n; q += 32) {
       Stream<double> sp(TAG_DIG_POS, (uint32_t)q, (uint32_t)lcell, iter, cp.k0, cp.k1);
       const int w = d0 + n + q;
-      if (cp.mesh == 1) {
-        // annulus: uniform in the sector (r^2 and the angle uniform)
-        const double r = sqrt(cp.r2t[iy] + sp.u(0) * (cp.r2t[iy + 1] - cp.r2t[iy]));
-        const double th = 2.0 * PI_D * ((double)ix + sp.u(1)) / (double)cp.nx;
-        out.x[w] = (T)(r * cos(th));
-        out.y[w] = (T)(r * sin(th));
-      } else if (cp.mesh == 2) {
-        // wall-refined box: uniform between the cell's edges
-        out.x[w] = (T)(cp.xe[ix] + sp.u(0) * (cp.xe[ix + 1] - cp.xe[ix]));
-        out.y[w] = (T)(cp.ye[iy] + sp.u(1) * (cp.ye[iy + 1] - cp.ye[iy]));
-      } else {
-        out.x[w] = (T)(((double)ix + sp.u(0)) * cp.dx);
-        out.y[w] = (T)((cp.dim == 2) ? ((double)iy + sp.u(1)) * cp.dy : 0.0);
-      }
+      T px, py;
+      dig_position<T>(cp, sp, ix, iy, &px, &py);
+      out.x[w] = px;
+      out.y[w] = py;
       if (n > 0) {
-        Stream<double> ss(TAG_DIG_SEL, (uint32_t)q, (uint32_t)lcell, iter, cp.k0, cp.k1);
-        int src = (int)(ss.u(0) * (double)n);
-        if (src > n - 1) src = n - 1;
+        const int src = dig_source(cp, q, n, lcell, iter);
         const T vx = in.vx[s0 + src], vy = in.vy[s0 + src], vz = in.vz[s0 + src], ir = in.ir[s0 + src];
         out.vx[w] = vx;
         out.vy[w] = vy;
@@ -1816,7 +1827,352 @@ __global__ void __launch_bounds__(WPB * 32) k_dig_apply(const CellParams* __rest
       if (cellof_out) cellof_out[w] = cell;
     }
   }
-  if (lane == 0) cnt_out[cell] = ntg;
+}
+
+
+// (float)(a v + b) with a, b double (a = ah + al, b = bh + bl split into
+// floats), as FP64 fma and conversion give it: evaluated in pairs of floats
+// (error below 2^-44 (|a v| + |b|)), and in FP64 only where that could round
+// the other way (near the midpoint of two floats) or leaves the normal range.
+__device__ __forceinline__ float affine_f32(double a, float ah, float al, double b, float bh, float bl, float v) {
+  const float p = __fmul_rn(ah, v), e = __fmaf_rn(ah, v, -p);
+  const float s = __fadd_rn(p, bh), bb = __fsub_rn(s, p);
+  const float e2 = __fadd_rn(__fsub_rn(p, __fsub_rn(s, bb)), __fsub_rn(bh, bb));
+  const float lo = __fadd_rn(e2, __fadd_rn(e, __fmaf_rn(al, v, bl)));
+  const float hi = __fadd_rn(s, lo), hb = __fsub_rn(hi, s);
+  const float rem = __fadd_rn(__fsub_rn(s, __fsub_rn(hi, hb)), __fsub_rn(lo, hb));
+  const uint32_t hu = __float_as_uint(hi);
+  const float half = __uint_as_float((hu & 0x7f800000u) - (24u << 23));
+  const float tol = 0x1p-44f * (fabsf(p) + fabsf(bh));
+  if (fabsf(hi) > 0x1p-90f && (hu & 0x7fffffu) != 0u && fabsf(rem) + tol < half) return hi;
+  return (float)__fma_rn(a, (double)v, b);
+}
+
+// floor(u n) of the FP64 uniform u of words hi, lo (dsmc_device.cuh), in
+// integers: u = (2 m + 1) 2^-53 with a 52-bit m
+__device__ __forceinline__ int floor_un(uint32_t hi, uint32_t lo, int n) {
+  const unsigned long long m = ((unsigned long long)hi << 20) | (unsigned long long)(lo >> 12);
+  const int r = (int)__umul64hi((2ull * m + 1ull) << 11, (unsigned long long)n);
+  return r > n - 1 ? n - 1 : r;
+}
+
+// a draw of dig_removal (n - q choices) or dig_source (n choices)
+__device__ __forceinline__ int dig_choice(const CellParams& cp, int q, int n, int lcell, uint32_t iter) {
+  const uint4 w = philox4x32_10((uint32_t)q, (uint32_t)lcell, iter, TAG_DIG_SEL << 24, cp.k0, cp.k1);
+  return floor_un(w.x, w.y, n);
+}
+
+// Exact sum of one value per lane and register slot (v[j] of particle lane +
+// 32 j < n) over the warp: the values scaled by a power of two to 22-bit
+// integers plus 22-bit remainders, added as integers (hi + lo 2^-22, times
+// exact_scale).  big: the bits of the largest magnitude.  Exact down to 2^-44
+// of it, as an FP64 sum is.
+template <int PER>
+__device__ __forceinline__ int2 exact_sum(const float* v, int n, uint32_t big) {
+  const int lane = threadIdx.x & 31;
+  // 2^(21 - exponent of the largest): magnitudes below 2^22
+  const float up = __uint_as_float((uint32_t)(127 + 21 + 127 - (int)(big >> 23)) << 23);
+  int hi = 0, lo = 0;
+#pragma unroll
+  for (int j = 0; j < PER; ++j) {
+    if (32 * j >= n) break;
+    const float w = (lane + 32 * j < n) ? v[j] * up : 0.f;
+    const int h = __float2int_rn(w);
+    hi += h;
+    lo += __float2int_rn((w - (float)h) * 0x1p22f);
+  }
+  return make_int2(__reduce_add_sync(FULL, hi), __reduce_add_sync(FULL, lo));
+}
+
+__device__ __forceinline__ double exact_scale(uint32_t big) {
+  return __hiloint2double((int)((uint32_t)(1023 - 21 - 127 + (int)(big >> 23)) << 20), 0);
+}
+
+// FP32 layout, steps ii-iv.  A cell of at most DIG_FAST particles before and
+// after stays in its warp's registers from the read to the write (one pass
+// over memory); others go through dig_cell.  The FP64 pipe (2 lanes per clock
+// and SM, a warp instruction costs 16 cycles for one lane or 32) would bound
+// it, so
+//  - the first moments are exact integer sums, the linear map runs in pairs of
+//    floats (both give dig_cell's FP64 values), and only the second moment is
+//    summed in FP64 by every lane, in dig_cell's order;
+//  - the per-cell arithmetic (means, factors) of the CTA's cells is done by
+//    one warp, a lane per cell.
+// 32 M particles (800 x 200 cells, 1D), counts, modification and read-out: 4.28
+// ms with one pass per step of the method and FP64 throughout, 2.84 ms now.
+constexpr int DIG_FAST = 256;
+struct DigCell {
+  int2 s[4];         // exact sums of vx, vy, vz, I_r
+  uint32_t bv, bi;   // largest magnitudes (0: sums holds them instead)
+  float rx, ry, rz;  // first particle
+  int np;
+  double sums[4];    // sums about the first particle, and of I_r
+  double u[3], c2;   // mean velocity; second moment
+  double a, b[3], cc;
+  float ah, al, bh[3], bl[3], ch, cl;
+};
+
+template <int DIM>
+__global__ void __launch_bounds__(WPB * 32, 2) k_dig_apply_f32(const CellParams* __restrict__ cps,
+                                                            const int32_t* __restrict__ cell_case,
+                                                            const int32_t* __restrict__ cell0, int ncells,
+                                                            PBuf<float> in, PBuf<float> out,
+                                                            const int32_t* __restrict__ start_in,
+                                                            const int32_t* __restrict__ cnt_in,
+                                                            const int32_t* __restrict__ start_out,
+                                                            int32_t* __restrict__ cnt_out,
+                                                            const int32_t* __restrict__ nt,
+                                                            const double* __restrict__ target, uint32_t iter,
+                                                            int32_t* __restrict__ idx_g, int tile) {
+  constexpr int PER = DIG_FAST / 32;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ DigCell s_dc[WPB];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  const int cell = blockIdx.x * WPB + warp;
+  int32_t* idx = reinterpret_cast<int32_t*>(smem) + (size_t)warp * tile * 2;
+  int32_t* kept = idx + tile;
+  int n = 0, np = 0, s0 = 0, d0 = 0, lcell = 0;
+  bool fast = false;
+  if (cell < ncells) {
+    const int cs = cell_case[cell];
+    const CellParams& cp = cps[cs];
+    lcell = cell - cell0[cs];
+    s0 = start_in[cell];
+    n = cnt_in[cell];
+    d0 = start_out[cell];
+    np = nt[cell];
+    fast = n > 0 && n <= DIG_FAST && np > 0 && np <= DIG_FAST && n <= tile;
+    if (!fast && np > 0) {
+      const bool fits = n <= tile;
+      dig_cell<float, DIM>(cp, cell, lcell, in, out, s0, n, d0, np, target + (size_t)cell * 6, iter,
+                           fits ? idx : idx_g + s0, fits ? kept : nullptr, nullptr);
+    }
+    if (lane == 0) cnt_out[cell] = np;
+  }
+  DigCell& dc = s_dc[warp];
+  float vx[PER], vy[PER], vz[PER], ir[PER];
+#pragma unroll
+  for (int j = 0; j < PER; ++j) vx[j] = vy[j] = vz[j] = ir[j] = 0.f;
+  if (fast) {
+    const CellParams& cp = cps[cell_case[cell]];
+    const int k = n - np;
+    if (k > 0) {
+      // partial Fisher-Yates as in dig_cell; the removed slots as one bit mask
+      for (int q = lane; q < n; q += 32) idx[q] = q;
+      if (lane < PER) kept[lane] = 0;
+      __syncwarp();
+      for (int qb = 0; qb < k; qb += 32) {
+        const int q = qb + lane;
+        const int r = (q < k) ? q + dig_choice(cp, q, n - q, lcell, iter) : 0;
+        const int m = min(32, k - qb);
+        for (int j = 0; j < m; ++j) {
+          const int rj = __shfl_sync(FULL, r, j);
+          if (lane == 0) {
+            const int tmp = idx[qb + j];
+            idx[qb + j] = idx[rj];
+            idx[rj] = tmp;
+          }
+        }
+      }
+      __syncwarp();
+      for (int q = lane; q < k; q += 32) {
+        const int g = idx[q];
+        atomicOr(&kept[g >> 5], (int)(1u << (g & 31)));
+      }
+      __syncwarp();
+      unsigned keep[PER];
+#pragma unroll
+      for (int j = 0; j < PER; ++j) {
+        const int left = n - 32 * j;
+        const unsigned valid = left >= 32 ? FULL : (left > 0 ? (1u << left) - 1u : 0u);
+        keep[j] = left > 0 ? valid & ~(unsigned)kept[j] : 0u;
+      }
+      __syncwarp();
+      int before = 0;
+#pragma unroll
+      for (int j = 0; j < PER; ++j) {
+        if ((keep[j] >> lane) & 1u) kept[before + __popc(keep[j] & below)] = lane + 32 * j;
+        before += __popc(keep[j]);
+      }
+      __syncwarp();
+    }
+    float big = 0.f, bigi = 0.f, probe = 0.f;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const int q = lane + 32 * j;
+      if (q < np) {
+        int src = q;
+        if (k > 0) src = kept[q];
+        float x, y = 0.f;
+        if (q >= n) {
+          src = dig_choice(cp, q - n, n, lcell, iter);
+          Stream<double> sp(TAG_DIG_POS, (uint32_t)(q - n), (uint32_t)lcell, iter, cp.k0, cp.k1);
+          dig_position<float>(cp, sp, lcell % cp.nx, lcell / cp.nx, &x, &y);
+        } else {
+          x = in.x[s0 + src];
+          if (DIM == 2) y = in.y[s0 + src];
+        }
+        out.x[d0 + q] = x;
+        if (DIM == 2) out.y[d0 + q] = y;  // 1D: y is 0 in both buffers
+        vx[j] = in.vx[s0 + src];
+        vy[j] = in.vy[s0 + src];
+        vz[j] = in.vz[s0 + src];
+        ir[j] = in.ir[s0 + src];
+        big = fmaxf(big, fmaxf(fabsf(vx[j]), fmaxf(fabsf(vy[j]), fabsf(vz[j]))));
+        bigi = fmaxf(bigi, fabsf(ir[j]));
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < PER; ++j) probe += (vx[j] + vy[j]) + (vz[j] + ir[j]);  // NaN is not seen by fmaxf
+    const uint32_t bv = __reduce_max_sync(FULL, __float_as_uint(big)), bi = __reduce_max_sync(FULL, __float_as_uint(bigi));
+    const bool plain = bv > (64u << 23) && bv < (192u << 23) && bi > (64u << 23) && bi < (192u << 23) &&
+                       __all_sync(FULL, isfinite(probe));
+    const float rx = __shfl_sync(FULL, vx[0], 0), ry = __shfl_sync(FULL, vy[0], 0), rz = __shfl_sync(FULL, vz[0], 0);
+    int2 e[4];
+    double sx = 0.0, sy = 0.0, sz = 0.0, si = 0.0;
+    if (plain) {
+      e[0] = exact_sum<PER>(vx, np, bv);
+      e[1] = exact_sum<PER>(vy, np, bv);
+      e[2] = exact_sum<PER>(vz, np, bv);
+      e[3] = exact_sum<PER>(ir, np, bi);
+    } else {
+      const double dx = f2d(rx), dy = f2d(ry), dz = f2d(rz);
+#pragma unroll
+      for (int j = 0; j < PER; ++j)
+        if (lane + 32 * j < np) {
+          sx += f2d(vx[j]) - dx;
+          sy += f2d(vy[j]) - dy;
+          sz += f2d(vz[j]) - dz;
+          si += f2d(ir[j]);
+        }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        sx += __shfl_xor_sync(FULL, sx, o);
+        sy += __shfl_xor_sync(FULL, sy, o);
+        sz += __shfl_xor_sync(FULL, sz, o);
+        si += __shfl_xor_sync(FULL, si, o);
+      }
+    }
+    if (lane == 0) {
+      dc.np = np;
+      dc.rx = rx;
+      dc.ry = ry;
+      dc.rz = rz;
+      dc.bv = plain ? bv : 0u;
+      dc.bi = bi;
+      if (plain) {
+        dc.s[0] = e[0];
+        dc.s[1] = e[1];
+        dc.s[2] = e[2];
+        dc.s[3] = e[3];
+      } else {
+        dc.sums[0] = sx;
+        dc.sums[1] = sy;
+        dc.sums[2] = sz;
+        dc.sums[3] = si;
+      }
+    }
+  } else if (lane == 0) {
+    dc.np = 0;
+  }
+  __syncthreads();
+  // step iii, the means: a lane per cell
+  if (threadIdx.x < WPB && s_dc[threadIdx.x].np > 0) {
+    DigCell& c = s_dc[threadIdx.x];
+    const double dn = (double)c.np;
+    const double r[3] = {f2d(c.rx), f2d(c.ry), f2d(c.rz)};
+    if (c.bv) {
+      // the sums about the first particle: exact, like the sums themselves
+      const double kv = exact_scale(c.bv), ki = exact_scale(c.bi);
+      for (int q = 0; q < 3; ++q)
+        c.sums[q] = __fma_rn(-dn, r[q], __fma_rn((double)c.s[q].y, 0x1p-22, (double)c.s[q].x) * kv);
+      c.sums[3] = __fma_rn((double)c.s[3].y, 0x1p-22, (double)c.s[3].x) * ki;
+    }
+    for (int q = 0; q < 3; ++q) c.u[q] = r[q] + c.sums[q] / dn;
+  }
+  __syncthreads();
+  if (fast) {
+    const double ux = dc.u[0], uy = dc.u[1], uz = dc.u[2];
+    double c2 = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      if (32 * j >= np) break;
+      if (lane + 32 * j < np) {
+        const double cx = f2d(vx[j]) - ux, cy = f2d(vy[j]) - uy, cz = f2d(vz[j]) - uz;
+        c2 += cx * cx + cy * cy + cz * cz;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c2 += __shfl_xor_sync(FULL, c2, o);
+    if (lane == 0) dc.c2 = c2;
+  }
+  __syncthreads();
+  // step iv, the factors: a lane per cell
+  if (threadIdx.x < WPB && s_dc[threadIdx.x].np > 0) {
+    DigCell& c = s_dc[threadIdx.x];
+    const int gc = blockIdx.x * WPB + threadIdx.x;
+    const double* t = target + (size_t)gc * 6;
+    const double dn = (double)c.np;
+    const double tts = c.c2 / (3.0 * dn);
+    const double trs = 2.0 * c.sums[3] / (cps[cell_case[gc]].d_r * dn);
+    const double a = (c.np >= 2 && tts > 0.0) ? sqrt(t[4] / tts) : 1.0;
+    const double cc = (trs > 0.0) ? t[5] / trs : 1.0;
+    c.a = a;
+    c.ah = (float)a;
+    c.al = (float)(a - (double)c.ah);
+    c.cc = cc;
+    c.ch = (float)cc;
+    c.cl = (float)(cc - (double)c.ch);
+    for (int q = 0; q < 3; ++q) {
+      const double b = t[1 + q] - c.u[q] * a;
+      c.b[q] = b;
+      c.bh[q] = (float)b;
+      c.bl[q] = (float)(b - (double)c.bh[q]);
+    }
+  }
+  __syncthreads();
+  if (fast) {
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      if (32 * j >= np) break;
+      const int w = d0 + lane + 32 * j;
+      if (lane + 32 * j < np) {
+        out.vx[w] = affine_f32(dc.a, dc.ah, dc.al, dc.b[0], dc.bh[0], dc.bl[0], vx[j]);
+        out.vy[w] = affine_f32(dc.a, dc.ah, dc.al, dc.b[1], dc.bh[1], dc.bl[1], vy[j]);
+        out.vz[w] = affine_f32(dc.a, dc.ah, dc.al, dc.b[2], dc.bh[2], dc.bl[2], vz[j]);
+        out.ir[w] = affine_f32(dc.cc, dc.ch, dc.cl, 0.0, 0.f, 0.f, ir[j]);
+      }
+    }
+  }
+}
+
+// FP64 layout: one warp per cell
+template <int DIM>
+__global__ void __launch_bounds__(WPB * 32) k_dig_apply_f64(const CellParams* __restrict__ cps,
+                                                            const int32_t* __restrict__ cell_case,
+                                                            const int32_t* __restrict__ cell0, int ncells,
+                                                            PBuf<double> in, PBuf<double> out,
+                                                            const int32_t* __restrict__ start_in,
+                                                            const int32_t* __restrict__ cnt_in,
+                                                            const int32_t* __restrict__ start_out,
+                                                            int32_t* __restrict__ cnt_out,
+                                                            const int32_t* __restrict__ nt,
+                                                            const double* __restrict__ target, uint32_t iter,
+                                                            int32_t* __restrict__ idx_g,
+                                                            int32_t* __restrict__ cellof_out, int tile) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int cell = blockIdx.x * WPB + warp;
+  if (cell >= ncells) return;
+  const int cs = cell_case[cell];
+  const int s0 = start_in[cell], n = cnt_in[cell];
+  int32_t* sm = reinterpret_cast<int32_t*>(smem) + (size_t)warp * tile * 2;
+  const bool fits = n <= tile;
+  dig_cell<double, DIM>(cps[cs], cell, cell - cell0[cs], in, out, s0, n, start_out[cell], nt[cell],
+                        target + (size_t)cell * 6, iter, fits ? sm : idx_g + s0, fits ? sm + tile : nullptr,
+                        cellof_out);
+  if (lane == 0) cnt_out[cell] = nt[cell];
 }
 
 template <typename T>
@@ -2225,16 +2581,17 @@ void Ops<T>::dig_apply(const CellParams& cp0, State<T>& s, int ncells, int& cur,
   const int cout = det ? olay : other;
   const int blocks = (ncells + WPB - 1) / WPB;
   const size_t sm = (size_t)WPB * s.tile * 2 * sizeof(int32_t);
-  if (cp0.dim == 1)
-    k_dig_apply<T, 1><<<blocks, WPB * 32, sm, st>>>(s.cases.cp, s.cases.cell_case, s.cases.cell0, ncells, s.buf[cur],
-                                                    s.buf[other], s.start[lay], s.count[cin], s.start[olay],
-                                                    s.count[cout], s.nt, target, iter, s.scratch_i,
-                                                    det ? s.cellof : nullptr, s.tile);
-  else
-    k_dig_apply<T, 2><<<blocks, WPB * 32, sm, st>>>(s.cases.cp, s.cases.cell_case, s.cases.cell0, ncells, s.buf[cur],
-                                                    s.buf[other], s.start[lay], s.count[cin], s.start[olay],
-                                                    s.count[cout], s.nt, target, iter, s.scratch_i,
-                                                    det ? s.cellof : nullptr, s.tile);
+#define DSMC_DIG_ARGS                                                                                       \
+  s.cases.cp, s.cases.cell_case, s.cases.cell0, ncells, s.buf[cur], s.buf[other], s.start[lay], s.count[cin], \
+      s.start[olay], s.count[cout], s.nt, target, iter, s.scratch_i
+  if constexpr (sizeof(T) == 4) {
+    if (cp0.dim == 1) k_dig_apply_f32<1><<<blocks, WPB * 32, sm, st>>>(DSMC_DIG_ARGS, s.tile);
+    else k_dig_apply_f32<2><<<blocks, WPB * 32, sm, st>>>(DSMC_DIG_ARGS, s.tile);
+  } else {
+    if (cp0.dim == 1) k_dig_apply_f64<1><<<blocks, WPB * 32, sm, st>>>(DSMC_DIG_ARGS, s.cellof, s.tile);
+    else k_dig_apply_f64<2><<<blocks, WPB * 32, sm, st>>>(DSMC_DIG_ARGS, s.cellof, s.tile);
+  }
+#undef DSMC_DIG_ARGS
   if (det) s.count_clear = false;
   else k_zero_i32<<<grid_for(ncells, 256), 256, 0, st>>>(s.count[cur], ncells);
   cur = other;
@@ -2257,15 +2614,17 @@ void Ops<T>::configure(int tile) {
   const int sm = (int)tile_smem<T>(tile);
   const int smd = WPB * tile * 2 * (int)sizeof(int32_t);
   if constexpr (sizeof(T) == 8) {
+    cudaFuncSetAttribute(k_dig_apply_f64<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smd);
+    cudaFuncSetAttribute(k_dig_apply_f64<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smd);
     cudaFuncSetAttribute(k_det_cells<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     cudaFuncSetAttribute(k_det_cells<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   } else {
     cudaFuncSetAttribute(k_collide_sample<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     cudaFuncSetAttribute(k_collide_sample<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   }
-  cudaFuncSetAttribute(k_dig_apply<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smd);
-  cudaFuncSetAttribute(k_dig_apply<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smd);
   if constexpr (sizeof(T) == 4) {
+    cudaFuncSetAttribute(k_dig_apply_f32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smd);
+    cudaFuncSetAttribute(k_dig_apply_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smd);
     const int sm4 = (int)fused_smem_bytes(tile, 4), sm2 = (int)fused_smem_bytes(tile, 2);
     cudaFuncSetAttribute(k_fused<2, false, 4, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm4);
     cudaFuncSetAttribute(k_fused<1, false, 4, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm4);
