@@ -1202,11 +1202,13 @@ int hot_mlp_grad(dsmc_handle* h, const double* dev_fields, const double* dev_hot
                  const uint8_t* dev_mask, float* host_grad, double* host_loss) {
   if (!h || !dev_fields || !dev_hot || !dev_kngll || !dev_mask) return set_err(h, DSMC_ERR_ARG, "bad arguments");
   mlp_data(h, dev_fields, dev_hot, dev_kngll, dev_mask);
+  // without a training cell the kernels give a zero loss and gradient: the
+  // count is looked at once they are queued
+  mlp_grad(h->mlp, h->ncells, h->stream);
   int n = 0;
   int r = mlp_count(h, &n);
   if (r) return r;
   if (n == 0) return set_err(h, DSMC_ERR_ARG, "hot_mlp_grad: no cell with mask = 1");
-  mlp_grad(h->mlp, h->ncells, h->stream);
   double loss = 0.0;
   cudaMemcpyAsync(&loss, h->mlp.scal, sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   if (host_grad)
@@ -1227,9 +1229,8 @@ int hot_mlp_train(dsmc_handle* h, const double* dev_fields, const double* dev_ho
   if (r) return r;
   if (n == 0) return set_err(h, DSMC_ERR_ARG, "hot_mlp_train: no cell with mask = 1");
   for (int k = 0; k < nsteps; ++k) {
-    mlp_grad(h->mlp, h->ncells, h->stream);
     h->mlp_t += 1;
-    mlp_adam(h->mlp, h->mlp_t, lr, h->stream);
+    mlp_train_step(h->mlp, h->ncells, h->mlp_t, lr, h->stream);
   }
   double loss = 0.0;
   cudaMemcpyAsync(&loss, h->mlp.scal, sizeof(double), cudaMemcpyDeviceToHost, h->stream);

@@ -165,7 +165,7 @@ int launch_synth2d(const CellParams& cp, const double* fields, const double* hot
 // HoT surrogate network (dsmc_mlp.cu): 12 -> 64 -> 64 -> 64 -> 5, tanh
 // hidden layers; parameters per layer: W (n_out x n_in, row major), then b.
 constexpr int MLP_NPARAM = 9477;
-constexpr int MLP_GRID = 304;  // largest grid of the forward/backward kernel
+constexpr int MLP_GRID = 152;  // largest grid of the training kernel (one CTA per SM)
 struct Mlp {
   float* theta;      // MLP_NPARAM FP32 master parameters
   uint16_t* wbf;     // MLP_NPARAM bfloat16 copies used by the kernels
@@ -190,8 +190,8 @@ void mlp_prepare(const Mlp& m, const CellParams* cp, const int32_t* cell_case, c
                  cudaStream_t st);
 // loss (scal[0]) and gradient (grad) of the weighted cells
 void mlp_grad(const Mlp& m, int ncells, cudaStream_t st);
-// one Adam step (step number t >= 1) and the bfloat16 copies
-void mlp_adam(const Mlp& m, int t, double lr, cudaStream_t st);
+// the same and one Adam step (step number t >= 1) with the bfloat16 copies
+void mlp_train_step(const Mlp& m, int ncells, int t, double lr, cudaStream_t st);
 // bfloat16 copies of the master parameters
 void mlp_to_bf16(const Mlp& m, cudaStream_t st);
 // network outputs, the HoT for the synthetic equations and the judge sums;

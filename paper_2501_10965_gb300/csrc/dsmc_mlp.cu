@@ -3,14 +3,9 @@
 // HoT it hands to the synthetic equations.  An extension: the paper takes
 // the higher-order terms of Eq. (hot_constitutive) from DSMC moments alone.
 //
-// Forward / backward: a CTA takes tiles of MLP_TILE cells.  The weights
-// (bfloat16 in global memory) are widened to FP32 in shared memory once per
-// CTA, rows padded by one word so that the threads of a warp, which work on
-// consecutive output neurons, read different banks.  A tile's activations of
-// all layers stay in shared memory for the backward pass.  Each thread owns
-// a fixed set of parameter gradients and sums its products over the tile's
-// cells, so the per-CTA sums need no atomics; the CTAs' sums are added in a
-// fixed order by a second kernel (the result does not depend on scheduling).
+// Training: see k_mlp_train.  The CTAs' gradient sums are added in a fixed
+// order by a second kernel (the result does not depend on scheduling), which
+// also takes the Adam step.
 #include <cmath>
 #include <cstdint>
 
@@ -24,31 +19,15 @@ namespace dsmc {
 
 namespace {
 
-constexpr int MLP_TILE = 32;
-constexpr int MLP_THREADS = 256;
 __host__ __device__ constexpr int nin(int k) { return k == 0 ? 12 : 64; }
 __host__ __device__ constexpr int nout(int k) { return k == 3 ? 5 : 64; }
 
-// offsets of W_k and b_k in the parameter vector, and of the padded W_k /
-// b_k in shared memory
+// offsets of W_k and b_k in the parameter vector
 __host__ __device__ constexpr int poff_w(int k) {
   return k == 0 ? 0 : poff_w(k - 1) + nin(k - 1) * nout(k - 1) + nout(k - 1);
 }
 __host__ __device__ constexpr int poff_b(int k) { return poff_w(k) + nin(k) * nout(k); }
-__host__ __device__ constexpr int soff_w(int k) {
-  return k == 0 ? 0 : soff_w(k - 1) + (nin(k - 1) + 1) * nout(k - 1) + nout(k - 1);
-}
-__host__ __device__ constexpr int soff_b(int k) { return soff_w(k) + (nin(k) + 1) * nout(k); }
-constexpr int SW_FLOATS = soff_b(3) + nout(3);
 static_assert(poff_b(3) + nout(3) == MLP_NPARAM, "parameter count");
-
-// shared memory: padded weights, gradient sums (training), activations
-// A0 (TILE x 12), A1..A3 (TILE x 64), output (TILE x 5), two delta buffers
-// (TILE x 64), cell weights (TILE)
-constexpr int ACT_FLOATS = MLP_TILE * (12 + 3 * 64 + 5 + 2 * 64 + 1);
-inline size_t fb_smem_bytes(bool train) {
-  return sizeof(float) * ((size_t)SW_FLOATS + (train ? (size_t)MLP_NPARAM : 0) + ACT_FLOATS);
-}
 
 __device__ __forceinline__ float bf16_to_f(uint16_t h) { return __uint_as_float((uint32_t)h << 16); }
 
@@ -163,168 +142,332 @@ __global__ void __launch_bounds__(128) k_mlp_data(const CellParams* __restrict__
   if ((threadIdx.x & 31) == 0 && used) atomicAdd(count, __popc(used));
 }
 
-template <int L, bool TANH>
-__device__ __forceinline__ void layer_fwd(const float* sw, const float* ain, float* aout) {
-  constexpr int ni = nin(L), no = nout(L);
-  const float* W = sw + soff_w(L);
-  const float* b = sw + soff_b(L);
-  for (int idx = threadIdx.x; idx < MLP_TILE * no; idx += blockDim.x) {
-    const int c = idx / no, j = idx % no;
-    const float* wr = W + j * (ni + 1);
-    const float* a = ain + c * ni;
-    float z = b[j];
-#pragma unroll 16
-    for (int i = 0; i < ni; ++i) z = fmaf(wr[i], a[i], z);
-    aout[idx] = TANH ? tanhf(z) : z;
+// ---------------------------------------------------------------------------
+// Loss and gradient (FP32 arithmetic on the bfloat16 weights).  A CTA of 256
+// threads takes tiles of 32 cells.  Bound by the FP32 pipe once the operands
+// come from shared memory in 16-byte loads: activations and deltas lie
+// feature by feature (row of a feature: the tile's 32 cells, padded to 36
+// words), so that
+//  - a layer's forward and delta products are 4 x 4 register tiles (4 cells, 4
+//    neurons a thread, two loads for 16 multiply-adds; 128 threads cover 32 x
+//    64), the weights kept in both orientations with the columns n, n + 16, n
+//    + 32, n + 48 of a thread adjacent;
+//  - a 64 x 64 weight gradient is a 4 x 4 tile per thread of all 256, summed
+//    over the cells four at a time, and stays in the thread's registers over
+//    all tiles of the CTA: no gradient in shared memory, no atomics.
+// The grid is one CTA per SM, and tiles of 32 keep the last round short: 12
+// 800 cells are 400 tiles, 3 rounds on 152 SMs.  12 800 cells: 108 us with
+// scalar products from shared memory and a gradient array there, 42 us.
+// ---------------------------------------------------------------------------
+constexpr int TR_TILE = 32;
+constexpr int TR_THREADS = 256;
+constexpr int TR_LD = TR_TILE + 4;
+// shared memory, floats
+constexpr int TR_W0T = 0;                       // [12][64], columns permuted
+constexpr int TR_W1T = TR_W0T + 12 * 64;        // [in 64][out 64]
+constexpr int TR_W2T = TR_W1T + 64 * 64;
+constexpr int TR_W1 = TR_W2T + 64 * 64;         // [out 64][in 64]
+constexpr int TR_W2 = TR_W1 + 64 * 64;
+constexpr int TR_W3 = TR_W2 + 64 * 64;          // [5][64], plain
+constexpr int TR_B = TR_W3 + 5 * 64;            // 3 x 64 + 8
+constexpr int TR_A0 = TR_B + 200;               // [12][36]
+constexpr int TR_A1 = TR_A0 + 12 * TR_LD;       // [64][36] x 3
+constexpr int TR_A2 = TR_A1 + 64 * TR_LD;
+constexpr int TR_A3 = TR_A2 + 64 * TR_LD;
+constexpr int TR_D3 = TR_A3 + 64 * TR_LD;       // [5][36]
+constexpr int TR_DA = TR_D3 + 5 * TR_LD;        // [64][36] x 2
+constexpr int TR_DB = TR_DA + 64 * TR_LD;
+constexpr int TR_WT = TR_DB + 64 * TR_LD;       // cell weights
+constexpr int TR_FLOATS = TR_WT + TR_TILE;
+inline size_t train_smem_bytes() { return sizeof(float) * (size_t)TR_FLOATS; }
+static_assert(TR_A0 % 4 == 0 && TR_D3 % 4 == 0 && TR_DA % 4 == 0 && TR_W1T % 4 == 0, "16-byte rows");
+
+// where column n of a 64-column row lies: the four columns of a thread (n & 15)
+// are adjacent
+__device__ __forceinline__ int perm64(int n) { return 4 * (n & 15) + (n >> 4); }
+
+// acc[c][n] += sum_i A[i][4 tc + c] W[i][column n of thread tn], i < K
+template <int K>
+__device__ __forceinline__ void tile_product(const float* A, const float* W, int tc, int tn, float (*acc)[4]) {
+#pragma unroll 8
+  for (int i = 0; i < K; ++i) {
+    const float4 a = *reinterpret_cast<const float4*>(A + i * TR_LD + 4 * tc);
+    const float4 w = *reinterpret_cast<const float4*>(W + i * 64 + 4 * tn);
+    const float av[4] = {a.x, a.y, a.z, a.w}, wv[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int n = 0; n < 4; ++n) acc[c][n] = fmaf(av[c], wv[n], acc[c][n]);
   }
 }
 
-// gradient sums of layer L from its output deltas d (TILE x no) and input
-// activations ain (TILE x ni); then, for L > 0, the deltas of the layer below
-// (through tanh' = 1 - a^2 of ain) into dnext
-template <int L>
-__device__ __forceinline__ void layer_bwd(const float* sw, float* g, const float* d, const float* ain,
-                                          float* dnext) {
-  constexpr int ni = nin(L), no = nout(L);
-  float* gW = g + poff_w(L);
-  float* gb = g + poff_b(L);
-  for (int idx = threadIdx.x; idx < no * ni; idx += blockDim.x) {
-    const int j = idx / ni, i = idx % ni;
-    float s = 0.f;
-#pragma unroll 8
-    for (int c = 0; c < MLP_TILE; ++c) s = fmaf(d[c * no + j], ain[c * ni + i], s);
-    gW[idx] += s;
+// out[n][c] = tanh(b[n] + sum_i W[n][i] A[i][c])
+template <int K>
+__device__ __forceinline__ void layer_forward(const float* A, const float* Wt, const float* b, float* out) {
+  if (threadIdx.x < 128) {
+    const int tn = threadIdx.x & 15, tc = threadIdx.x >> 4;
+    float acc[4][4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      const float bn = b[tn + 16 * n];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[c][n] = bn;
+    }
+    tile_product<K>(A, Wt, tc, tn, acc);
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+      *reinterpret_cast<float4*>(out + (tn + 16 * n) * TR_LD + 4 * tc) =
+          make_float4(tanhf(acc[0][n]), tanhf(acc[1][n]), tanhf(acc[2][n]), tanhf(acc[3][n]));
   }
-  for (int j = threadIdx.x; j < no; j += blockDim.x) {
-    float s = 0.f;
-    for (int c = 0; c < MLP_TILE; ++c) s += d[c * no + j];
-    gb[j] += s;
-  }
-  if (L > 0) {
-    const float* W = sw + soff_w(L);
-    for (int idx = threadIdx.x; idx < MLP_TILE * ni; idx += blockDim.x) {
-      const int c = idx / ni, i = idx % ni;
-      float s = 0.f;
-#pragma unroll 8
-      for (int j = 0; j < no; ++j) s = fmaf(d[c * no + j], W[j * (ni + 1) + i], s);
-      const float a = ain[idx];
-      dnext[idx] = s * (1.f - a * a);
+}
+
+// deltas of the layer below: out[i][c] = (1 - A[i][c]^2) sum_j W[j][i] D[j][c]
+__device__ __forceinline__ void layer_delta(const float* D, const float* W, const float* A, float* out) {
+  if (threadIdx.x < 128) {
+    const int tn = threadIdx.x & 15, tc = threadIdx.x >> 4;
+    float acc[4][4];
+#pragma unroll
+    for (int n = 0; n < 4; ++n)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[c][n] = 0.f;
+    tile_product<64>(D, W, tc, tn, acc);
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      const int o = (tn + 16 * n) * TR_LD + 4 * tc;
+      const float4 a = *reinterpret_cast<const float4*>(A + o);
+      *reinterpret_cast<float4*>(out + o) =
+          make_float4(acc[0][n] * (1.f - a.x * a.x), acc[1][n] * (1.f - a.y * a.y), acc[2][n] * (1.f - a.z * a.z),
+                      acc[3][n] * (1.f - a.w * a.w));
     }
   }
 }
 
-template <bool TRAIN>
-__global__ void __launch_bounds__(MLP_THREADS) k_mlp_fb(const uint16_t* __restrict__ wbf, const float* __restrict__ X,
-                                                        const float* __restrict__ Y, const float* __restrict__ wc,
-                                                        const int32_t* __restrict__ count, int ncells,
-                                                        float* __restrict__ partial, double* __restrict__ part_loss,
-                                                        float* __restrict__ out) {
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, float s) {
+  s = fmaf(a.x, b.x, s);
+  s = fmaf(a.y, b.y, s);
+  s = fmaf(a.z, b.z, s);
+  return fmaf(a.w, b.w, s);
+}
+
+__device__ __forceinline__ float4 row4(const float* M, int row, int c) {
+  return *reinterpret_cast<const float4*>(M + row * TR_LD + c);
+}
+
+// g[m][n] += sum_c D[tm + 16 m][c] A[tn + 16 n][c] of a 64 x 64 layer
+__device__ __forceinline__ void weight_gradient(const float* D, const float* A, float (*g)[4]) {
+  const int tn = threadIdx.x & 15, tm = threadIdx.x >> 4;
+#pragma unroll 2
+  for (int c = 0; c < TR_TILE; c += 4) {
+    float4 d[4], a[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      d[k] = row4(D, tm + 16 * k, c);
+      a[k] = row4(A, tn + 16 * k, c);
+    }
+#pragma unroll
+    for (int m = 0; m < 4; ++m)
+#pragma unroll
+      for (int n = 0; n < 4; ++n) g[m][n] = dot4(d[m], a[n], g[m][n]);
+  }
+}
+
+__device__ __forceinline__ float row_sum(const float* M, int row, float s) {
+#pragma unroll
+  for (int c = 0; c < TR_TILE; c += 4) {
+    const float4 v = row4(M, row, c);
+    s += (v.x + v.y) + (v.z + v.w);
+  }
+  return s;
+}
+
+__global__ void __launch_bounds__(TR_THREADS) k_mlp_train(const uint16_t* __restrict__ wbf,
+                                                          const float* __restrict__ X, const float* __restrict__ Y,
+                                                          const float* __restrict__ wc,
+                                                          const int32_t* __restrict__ count, int ncells,
+                                                          float* __restrict__ partial,
+                                                          double* __restrict__ part_loss) {
   extern __shared__ __align__(16) float sm[];
-  float* sw = sm;
-  float* g = sw + SW_FLOATS;
-  float* a0 = g + (TRAIN ? MLP_NPARAM : 0);
-  float* a1 = a0 + MLP_TILE * 12;
-  float* a2 = a1 + MLP_TILE * 64;
-  float* a3 = a2 + MLP_TILE * 64;
-  float* ao = a3 + MLP_TILE * 64;
-  float* d0 = ao + MLP_TILE * 5;
-  float* d1 = d0 + MLP_TILE * 64;
-  float* wt = d1 + MLP_TILE * 64;
-  __shared__ double red[MLP_THREADS];
-  // widen the weights into padded rows
-  for (int k = 0; k < 4; ++k) {
-    const int ni = nin(k), no = nout(k);
-    for (int idx = threadIdx.x; idx < no * ni; idx += blockDim.x) {
-      const int j = idx / ni, i = idx % ni;
-      sw[soff_w(k) + j * (ni + 1) + i] = bf16_to_f(wbf[poff_w(k) + idx]);
-    }
-    for (int j = threadIdx.x; j < no; j += blockDim.x) sw[soff_b(k) + j] = bf16_to_f(wbf[poff_b(k) + j]);
+  __shared__ double red[TR_THREADS / 32];
+  const int tid = threadIdx.x;
+  // weights, widened
+  for (int q = tid; q < 12 * 64; q += TR_THREADS) {
+    const int j = q / 12, i = q % 12;
+    sm[TR_W0T + i * 64 + perm64(j)] = bf16_to_f(wbf[poff_w(0) + q]);
   }
-  if (TRAIN)
-    for (int q = threadIdx.x; q < MLP_NPARAM; q += blockDim.x) g[q] = 0.f;
-  const float inv_n = TRAIN ? 1.f / (5.f * (float)max(*count, 1)) : 0.f;
+  for (int q = tid; q < 64 * 64; q += TR_THREADS) {
+    const int j = q >> 6, i = q & 63;
+    const float w1 = bf16_to_f(wbf[poff_w(1) + q]), w2 = bf16_to_f(wbf[poff_w(2) + q]);
+    sm[TR_W1T + i * 64 + perm64(j)] = w1;
+    sm[TR_W2T + i * 64 + perm64(j)] = w2;
+    sm[TR_W1 + j * 64 + perm64(i)] = w1;
+    sm[TR_W2 + j * 64 + perm64(i)] = w2;
+  }
+  for (int q = tid; q < 5 * 64; q += TR_THREADS) sm[TR_W3 + q] = bf16_to_f(wbf[poff_w(3) + q]);
+  if (tid < 64) {
+    sm[TR_B + tid] = bf16_to_f(wbf[poff_b(0) + tid]);
+    sm[TR_B + 64 + tid] = bf16_to_f(wbf[poff_b(1) + tid]);
+    sm[TR_B + 128 + tid] = bf16_to_f(wbf[poff_b(2) + tid]);
+    if (tid < 5) sm[TR_B + 192 + tid] = bf16_to_f(wbf[poff_b(3) + tid]);
+  }
+  const int tn = tid & 15, tm = tid >> 4;
+  float g0[4] = {0.f, 0.f, 0.f, 0.f}, g1[4][4], g2[4][4], g3[2] = {0.f, 0.f};
+  float gb[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+#pragma unroll
+    for (int n = 0; n < 4; ++n) g1[m][n] = g2[m][n] = 0.f;
+  const float inv_n = 1.f / (5.f * (float)max(*count, 1));
   double lsum = 0.0;
   __syncthreads();
-  const int ntiles = (ncells + MLP_TILE - 1) / MLP_TILE;
+  const int ntiles = (ncells + TR_TILE - 1) / TR_TILE;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int c0 = t * MLP_TILE;
-    for (int idx = threadIdx.x; idx < MLP_TILE * 12; idx += blockDim.x) {
-      const int c = c0 + idx / 12;
-      a0[idx] = (c < ncells) ? X[(size_t)c0 * 12 + idx] : 0.f;
+    const int c0 = t * TR_TILE;
+    for (int q = tid; q < TR_TILE * 12; q += TR_THREADS) {
+      const int c = q / 12, i = q % 12;
+      sm[TR_A0 + i * TR_LD + c] = (c0 + c < ncells) ? X[(size_t)c0 * 12 + q] : 0.f;
     }
-    for (int c = threadIdx.x; c < MLP_TILE; c += blockDim.x) wt[c] = (c0 + c < ncells) ? wc[c0 + c] : 0.f;
+    if (tid < TR_TILE) sm[TR_WT + tid] = (c0 + tid < ncells) ? wc[c0 + tid] : 0.f;
     __syncthreads();
-    layer_fwd<0, true>(sw, a0, a1);
+    layer_forward<12>(sm + TR_A0, sm + TR_W0T, sm + TR_B, sm + TR_A1);
     __syncthreads();
-    layer_fwd<1, true>(sw, a1, a2);
+    layer_forward<64>(sm + TR_A1, sm + TR_W1T, sm + TR_B + 64, sm + TR_A2);
     __syncthreads();
-    layer_fwd<2, true>(sw, a2, a3);
+    layer_forward<64>(sm + TR_A2, sm + TR_W2T, sm + TR_B + 128, sm + TR_A3);
     __syncthreads();
-    layer_fwd<3, false>(sw, a3, ao);
+    // output layer and the deltas of the mean squared error over the weighted
+    // cells: a thread per (output, cell)
+    if (tid < 5 * TR_TILE) {
+      const int j = tid / TR_TILE, c = tid % TR_TILE;
+      float z[4] = {sm[TR_B + 192 + j], 0.f, 0.f, 0.f};
+#pragma unroll 4
+      for (int i = 0; i < 64; i += 4)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) z[k] = fmaf(sm[TR_W3 + j * 64 + i + k], sm[TR_A3 + (i + k) * TR_LD + c], z[k]);
+      const float y = (c0 + c < ncells) ? Y[(size_t)(c0 + c) * 5 + j] : 0.f;
+      const float r = ((z[0] + z[1]) + (z[2] + z[3]) - y) * sm[TR_WT + c];
+      lsum += (double)r * (double)r;
+      sm[TR_D3 + j * TR_LD + c] = 2.f * r * inv_n;
+    }
     __syncthreads();
-    if (!TRAIN) {
-      for (int idx = threadIdx.x; idx < MLP_TILE * 5; idx += blockDim.x)
-        if (c0 + idx / 5 < ncells) out[(size_t)c0 * 5 + idx] = ao[idx];
-    } else {
-      // output deltas of the mean squared error over the weighted cells
-      for (int idx = threadIdx.x; idx < MLP_TILE * 5; idx += blockDim.x) {
-        const int c = idx / 5;
-        const float y = (c0 + c < ncells) ? Y[(size_t)c0 * 5 + idx] : 0.f;
-        const float r = (ao[idx] - y) * wt[c];
-        lsum += (double)r * (double)r;
-        d0[idx] = 2.f * r * inv_n;
+    // layer 3: gradient, bias, deltas of layer 2's output
+    {
+      const int j = tid >> 6, i = tid & 63;
+#pragma unroll
+      for (int c = 0; c < TR_TILE; c += 4) {
+        const float4 a = row4(sm + TR_A3, i, c);
+        g3[0] = dot4(row4(sm + TR_D3, j, c), a, g3[0]);
+        if (tid < 64) g3[1] = dot4(row4(sm + TR_D3, 4, c), a, g3[1]);
       }
-      __syncthreads();
-      layer_bwd<3>(sw, g, d0, a3, d1);
-      __syncthreads();
-      layer_bwd<2>(sw, g, d1, a2, d0);
-      __syncthreads();
-      layer_bwd<1>(sw, g, d0, a1, d1);
-      __syncthreads();
-      layer_bwd<0>(sw, g, d1, a0, nullptr);
+      if (tid < 5) gb[3] = row_sum(sm + TR_D3, tid, gb[3]);
+      for (int q = tid; q < 64 * (TR_TILE / 4); q += TR_THREADS) {
+        const int n = q >> 3, c = 4 * (q & 7);
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 5; ++k) {
+          const float w = sm[TR_W3 + k * 64 + n];
+          const float4 d = row4(sm + TR_D3, k, c);
+          s.x = fmaf(d.x, w, s.x);
+          s.y = fmaf(d.y, w, s.y);
+          s.z = fmaf(d.z, w, s.z);
+          s.w = fmaf(d.w, w, s.w);
+        }
+        const float4 a = row4(sm + TR_A3, n, c);
+        *reinterpret_cast<float4*>(sm + TR_DA + n * TR_LD + c) =
+            make_float4(s.x * (1.f - a.x * a.x), s.y * (1.f - a.y * a.y), s.z * (1.f - a.z * a.z),
+                        s.w * (1.f - a.w * a.w));
+      }
     }
     __syncthreads();
-  }
-  if (TRAIN) {
-    for (int q = threadIdx.x; q < MLP_NPARAM; q += blockDim.x) partial[(size_t)blockIdx.x * MLP_NPARAM + q] = g[q];
-    red[threadIdx.x] = lsum;
+    weight_gradient(sm + TR_DA, sm + TR_A2, g2);
+    if (tid < 64) gb[2] = row_sum(sm + TR_DA, tid, gb[2]);
+    layer_delta(sm + TR_DA, sm + TR_W2, sm + TR_A2, sm + TR_DB);
     __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-      if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-      __syncthreads();
+    weight_gradient(sm + TR_DB, sm + TR_A1, g1);
+    if (tid < 64) gb[1] = row_sum(sm + TR_DB, tid, gb[1]);
+    layer_delta(sm + TR_DB, sm + TR_W1, sm + TR_A1, sm + TR_DA);
+    __syncthreads();
+    if (tn < 12) {
+#pragma unroll
+      for (int c = 0; c < TR_TILE; c += 4) {
+        const float4 a = row4(sm + TR_A0, tn, c);
+#pragma unroll
+        for (int m = 0; m < 4; ++m) g0[m] = dot4(row4(sm + TR_DA, tm + 16 * m, c), a, g0[m]);
+      }
     }
-    if (threadIdx.x == 0) part_loss[blockIdx.x] = red[0];
+    if (tid < 64) gb[0] = row_sum(sm + TR_DA, tid, gb[0]);
+    __syncthreads();
   }
-}
-
-// the CTAs' gradient sums in block order; the loss
-__global__ void k_mlp_reduce(const float* __restrict__ partial, const double* __restrict__ part_loss, int nblk,
-                             const int32_t* __restrict__ count, float* __restrict__ grad, double* __restrict__ scal) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < MLP_NPARAM) {
-    float s = 0.f;
-    for (int b = 0; b < nblk; ++b) s += partial[(size_t)b * MLP_NPARAM + q];
-    grad[q] = s;
+  float* out = partial + (size_t)blockIdx.x * MLP_NPARAM;
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    if (tn < 12) out[poff_w(0) + (tm + 16 * m) * 12 + tn] = g0[m];
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      out[poff_w(1) + (tm + 16 * m) * 64 + tn + 16 * n] = g1[m][n];
+      out[poff_w(2) + (tm + 16 * m) * 64 + tn + 16 * n] = g2[m][n];
+    }
   }
-  if (q == 0) {
+  out[poff_w(3) + tid] = g3[0];
+  if (tid < 64) {
+    out[poff_w(3) + 256 + tid] = g3[1];
+    out[poff_b(0) + tid] = gb[0];
+    out[poff_b(1) + tid] = gb[1];
+    out[poff_b(2) + tid] = gb[2];
+    if (tid < 5) out[poff_b(3) + tid] = gb[3];
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
+  if ((tid & 31) == 0) red[tid >> 5] = lsum;
+  __syncthreads();
+  if (tid == 0) {
     double l = 0.0;
-    for (int b = 0; b < nblk; ++b) l += part_loss[b];
-    scal[0] = l / (5.0 * (double)max(*count, 1));
+    for (int k = 0; k < TR_THREADS / 32; ++k) l += red[k];
+    part_loss[blockIdx.x] = l;
   }
 }
 
-__global__ void k_mlp_adam(float* __restrict__ theta, float* __restrict__ m, float* __restrict__ v,
-                           const float* __restrict__ grad, uint16_t* __restrict__ wbf, float c1, float c2, float lr) {
-  const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q >= MLP_NPARAM) return;
-  const float gq = grad[q];
-  const float mq = 0.9f * m[q] + 0.1f * gq;
-  const float vq = 0.999f * v[q] + 0.001f * gq * gq;
-  m[q] = mq;
-  v[q] = vq;
-  const float th = theta[q] - lr * (mq / c1) / (sqrtf(vq / c2) + 1e-8f);
-  theta[q] = th;
-  wbf[q] = __bfloat16_as_ushort(__float2bfloat16_rn(th));
+// The CTAs' gradient sums in a fixed order (32 parameters per CTA, eight
+// threads each on every eighth sum); the loss; with ADAM the step.  A thread
+// per parameter over all sums took 24 us at 12 800 cells: REDUCE_US.
+template <bool ADAM>
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ partial,
+                                                    const double* __restrict__ part_loss, int nblk,
+                                                    const int32_t* __restrict__ count, float* __restrict__ grad,
+                                                    double* __restrict__ scal, float* __restrict__ theta,
+                                                    float* __restrict__ m, float* __restrict__ v,
+                                                    uint16_t* __restrict__ wbf, float c1, float c2, float lr) {
+  __shared__ float s[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int q = blockIdx.x * 32 + lane;
+  float a = 0.f;
+  if (q < MLP_NPARAM) {
+#pragma unroll 4
+    for (int b = w; b < nblk; b += 8) a += partial[(size_t)b * MLP_NPARAM + q];
+  }
+  s[w][lane] = a;
+  __syncthreads();
+  if (w == 0 && q < MLP_NPARAM) {
+    float gq = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) gq += s[k][lane];
+    grad[q] = gq;
+    if (ADAM) {
+      const float mq = 0.9f * m[q] + 0.1f * gq;
+      const float vq = 0.999f * v[q] + 0.001f * gq * gq;
+      m[q] = mq;
+      v[q] = vq;
+      const float th = theta[q] - lr * (mq / c1) / (sqrtf(vq / c2) + 1e-8f);
+      theta[q] = th;
+      wbf[q] = __bfloat16_as_ushort(__float2bfloat16_rn(th));
+    }
+  }
+  if (blockIdx.x == 0 && w == 1) {
+    double l = 0.0;
+    for (int b = lane; b < nblk; b += 32) l += part_loss[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) scal[0] = l / (5.0 * (double)max(*count, 1));
+  }
 }
 
 __global__ void k_mlp_bf16(const float* __restrict__ theta, uint16_t* __restrict__ wbf) {
@@ -343,6 +486,7 @@ __global__ void k_mlp_bf16(const float* __restrict__ theta, uint16_t* __restrict
 // rows padded so that the fragment loads of a warp hit 32 distinct banks.
 // ---------------------------------------------------------------------------
 constexpr int TC_WARPS = 4;
+constexpr int TC_GRID = 304;      // largest grid
 constexpr int TC_K0 = 16;        // the 12 inputs padded to one k-slice
 constexpr int TC_LD0 = 12;       // words per row of the padded layer-0 weights (8 used)
 constexpr int TC_LD = 36;        // words per row of the 64-input weights (32 used)
@@ -593,13 +737,13 @@ __global__ void __launch_bounds__(256) k_mlp_hot(int ncells, const float* __rest
 
 inline int blocks_for(int n, int t) { return (n + t - 1) / t; }
 
-void configure_fb() {
-  static bool configured = false;
-  if (!configured) {
-    cudaFuncSetAttribute(k_mlp_fb<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fb_smem_bytes(true));
-    cudaFuncSetAttribute(k_mlp_fb<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fb_smem_bytes(false));
-    configured = true;
-  }
+int launch_train(const Mlp& m, int ncells, cudaStream_t st) {
+  cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)train_smem_bytes());
+  const int ntiles = blocks_for(ncells, TR_TILE);
+  const int grid = ntiles < MLP_GRID ? ntiles : MLP_GRID;
+  k_mlp_train<<<grid, TR_THREADS, train_smem_bytes(), st>>>(m.wbf, m.X, m.Y, m.w, m.count, ncells, m.partial,
+                                                            m.part_loss);
+  return grid;
 }
 
 }  // namespace
@@ -613,17 +757,16 @@ void mlp_prepare(const Mlp& m, const CellParams* cp, const int32_t* cell_case, c
 }
 
 void mlp_grad(const Mlp& m, int ncells, cudaStream_t st) {
-  configure_fb();
-  const int ntiles = blocks_for(ncells, MLP_TILE);
-  const int grid = ntiles < MLP_GRID ? ntiles : MLP_GRID;
-  k_mlp_fb<true><<<grid, MLP_THREADS, fb_smem_bytes(true), st>>>(m.wbf, m.X, m.Y, m.w, m.count, ncells, m.partial,
-                                                                  m.part_loss, m.out);
-  k_mlp_reduce<<<blocks_for(MLP_NPARAM, 256), 256, 0, st>>>(m.partial, m.part_loss, grid, m.count, m.grad, m.scal);
+  const int grid = launch_train(m, ncells, st);
+  k_mlp_reduce<false><<<blocks_for(MLP_NPARAM, 32), 256, 0, st>>>(m.partial, m.part_loss, grid, m.count, m.grad, m.scal,
+                                                                  m.theta, m.m, m.v, m.wbf, 1.f, 1.f, 0.f);
 }
 
-void mlp_adam(const Mlp& m, int t, double lr, cudaStream_t st) {
+void mlp_train_step(const Mlp& m, int ncells, int t, double lr, cudaStream_t st) {
+  const int grid = launch_train(m, ncells, st);
   const float c1 = (float)(1.0 - pow(0.9, t)), c2 = (float)(1.0 - pow(0.999, t));
-  k_mlp_adam<<<blocks_for(MLP_NPARAM, 256), 256, 0, st>>>(m.theta, m.m, m.v, m.grad, m.wbf, c1, c2, (float)lr);
+  k_mlp_reduce<true><<<blocks_for(MLP_NPARAM, 32), 256, 0, st>>>(m.partial, m.part_loss, grid, m.count, m.grad, m.scal,
+                                                                 m.theta, m.m, m.v, m.wbf, c1, c2, (float)lr);
 }
 
 void mlp_to_bf16(const Mlp& m, cudaStream_t st) {
@@ -634,7 +777,7 @@ void mlp_apply(const Mlp& m, int ncells, const double* hot, double* hot_out, cud
                const int32_t* group, double z, int min_samples, double rel) {
   // inference on the tensor cores (bfloat16 weights and activations, FP32 sums)
   const int tiles = blocks_for(ncells, 16);
-  const int grid = blocks_for(tiles, TC_WARPS) < MLP_GRID ? blocks_for(tiles, TC_WARPS) : MLP_GRID;
+  const int grid = blocks_for(tiles, TC_WARPS) < TC_GRID ? blocks_for(tiles, TC_WARPS) : TC_GRID;
   k_mlp_fwd_tc<<<grid, TC_WARPS * 32, tc_smem_bytes(), st>>>(m.wbf, m.theta, m.X, ncells, m.out);
   cudaMemsetAsync(m.scal + 2, 0, 3 * sizeof(double), st);
   const int hb = blocks_for(ncells, 256) < 1024 ? blocks_for(ncells, 256) : 1024;
