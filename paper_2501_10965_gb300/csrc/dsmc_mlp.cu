@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_mlp_train(const uint16_t* __rest
 
 // The CTAs' gradient sums in a fixed order (32 parameters per CTA, eight
 // threads each on every eighth sum); the loss; with ADAM the step.  A thread
-// per parameter over all sums took 24 us at 12 800 cells: REDUCE_US.
+// per parameter over all sums took 24 us at 12 800 cells, this 5 us.
 template <bool ADAM>
 __global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ partial,
                                                     const double* __restrict__ part_loss, int nblk,
