@@ -37,7 +37,7 @@ __device__ __forceinline__ float bf16_to_f(uint16_t h) { return __uint_as_float(
 // The FP64 pipe bounds it (2 lanes per clock and SM): the divisions by the
 // cell's own scales are one reciprocal each, the y gradients of a 1D case
 // (zero) are not formed.  The count is added once per warp.
-// 160 000 cells (1D): 236 us before, 98 us now.
+// 160 000 cells (1D): 236 us before, 61 us now.
 __global__ void __launch_bounds__(128) k_mlp_data(const CellParams* __restrict__ cps,
                            const int32_t* __restrict__ cell_case,
                            const int32_t* __restrict__ cell0, int ncells, const double* __restrict__ F,
@@ -65,7 +65,9 @@ __global__ void __launch_bounds__(128) k_mlp_data(const CellParams* __restrict__
       ok = rho > 0.0 && tt > 0.0 && tr > 0.0 && isfinite(T);
       if (ok) {
         const bool one = cp.dim == 1;
-        const double mu = cp.mu_ref * pow(T, cp.omega);
+        // T^omega as exp(omega log T), within a few ulp of 64 bits; the inputs
+        // are rounded to 32
+        const double mu = cp.mu_ref * exp(cp.omega * log(T));
         const double sq = sqrt(T), iT = 1.0 / T, irho = 1.0 / rho, isq = sq * iT;
         // lambda / norm of rho; u_x, u_y; T_t, T_r
         const double lam = mu * irho * isq * 1.2533141373155003;  // sqrt(pi / 2)
@@ -484,9 +486,11 @@ __global__ void k_mlp_bf16(const float* __restrict__ theta, uint16_t* __restrict
 // is the operand fragment of one 16-column k-slice).  A warp takes 16 cells
 // at a time; the CTA's warps share the weights, staged in shared memory in
 // rows padded so that the fragment loads of a warp hit 32 distinct banks.
+// 160 000 cells: 48 us with 4 warps a CTA and two CTAs an SM, 42 us with 8 and
+// three (the latency of a tile's chain of products bounds it).
 // ---------------------------------------------------------------------------
-constexpr int TC_WARPS = 4;
-constexpr int TC_GRID = 304;      // largest grid
+constexpr int TC_WARPS = 8;
+constexpr int TC_GRID = 3 * 152;  // largest grid: 24 warps an SM share three copies of the weights
 constexpr int TC_K0 = 16;        // the 12 inputs padded to one k-slice
 constexpr int TC_LD0 = 12;       // words per row of the padded layer-0 weights (8 used)
 constexpr int TC_LD = 36;        // words per row of the 64-input weights (32 used)
