@@ -1491,11 +1491,16 @@ __global__ void k_rebin_ovf(const Ovf ov, int ovf_cap, PBuf<float> out, const in
 // export / import
 // ---------------------------------------------------------------------------
 // float -> double by integer operations where the value is normal (the
-// conversion instruction runs on the FP64 pipe at 2 lanes per clock and SM)
+// conversion instruction runs on the FP64 pipe at 2 lanes per clock and SM).
+// The rare cases are calls: inlined, they were executed under a predicate for
+// every value, at the FP64 pipe's cost.
+static __device__ __noinline__ double f2d_rare(float v) { return (double)v; }
 __device__ __forceinline__ double f2d(float v) {
   const uint32_t u = __float_as_uint(v), e = u & 0x7f800000u;
-  if (e == 0u || e == 0x7f800000u) return (double)v;
-  return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(u << 29));
+  const bool zero = (u << 1) == 0u;
+  if (!zero && (e == 0u || e == 0x7f800000u)) return f2d_rare(v);
+  const uint32_t hi = zero ? u : (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u);
+  return __hiloint2double((int)hi, (int)(u << 29));
 }
 __device__ __forceinline__ double to_double(float v) { return f2d(v); }
 __device__ __forceinline__ double to_double(double v) { return v; }
@@ -1834,6 +1839,9 @@ __device__ void dig_cell(const CellParams& cp, int cell, int lcell, const PBuf<T
 // floats), as FP64 fma and conversion give it: evaluated in pairs of floats
 // (error below 2^-44 (|a v| + |b|)), and in FP64 only where that could round
 // the other way (near the midpoint of two floats) or leaves the normal range.
+static __device__ __noinline__ float affine_rare(double a, double b, float v) {
+  return (float)__fma_rn(a, (double)v, b);
+}
 __device__ __forceinline__ float affine_f32(double a, float ah, float al, double b, float bh, float bl, float v) {
   const float p = __fmul_rn(ah, v), e = __fmaf_rn(ah, v, -p);
   const float s = __fadd_rn(p, bh), bb = __fsub_rn(s, p);
@@ -1845,7 +1853,7 @@ __device__ __forceinline__ float affine_f32(double a, float ah, float al, double
   const float half = __uint_as_float((hu & 0x7f800000u) - (24u << 23));
   const float tol = 0x1p-44f * (fabsf(p) + fabsf(bh));
   if (fabsf(hi) > 0x1p-90f && (hu & 0x7fffffu) != 0u && fabsf(rem) + tol < half) return hi;
-  return (float)__fma_rn(a, (double)v, b);
+  return affine_rare(a, b, v);
 }
 
 // floor(u n) of the FP64 uniform u of words hi, lo (dsmc_device.cuh), in
@@ -1899,7 +1907,7 @@ __device__ __forceinline__ double exact_scale(uint32_t big) {
 //  - the per-cell arithmetic (means, factors) of the CTA's cells is done by
 //    one warp, a lane per cell.
 // 32 M particles (800 x 200 cells, 1D), counts, modification and read-out: 4.28
-// ms with one pass per step of the method and FP64 throughout, 2.84 ms now.
+// ms with one pass per step of the method and FP64 throughout, 2.50 ms now.
 constexpr int DIG_FAST = 256;
 struct DigCell {
   int2 s[4];         // exact sums of vx, vy, vz, I_r
