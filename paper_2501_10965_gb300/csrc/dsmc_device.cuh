@@ -94,9 +94,11 @@ __device__ __forceinline__ uint4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_
   return make_uint4(c0, c1, c2, c3);
 }
 
+// (m + 1/2) 2^-52 for the 52-bit m of the two words, exactly: m as the mantissa
+// of 1 + m 2^-52, less 1 - 2^-53 (one FP64 operation; the conversion of a
+// 64-bit integer and the two operations after it all run on the FP64 pipe)
 __device__ __forceinline__ double u01_from_words(uint32_t hi, uint32_t lo) {
-  const unsigned long long m = ((unsigned long long)hi << 20) | (unsigned long long)(lo >> 12);
-  return ((double)m + 0.5) * 0x1p-52;
+  return __hiloint2double((int)(0x3ff00000u | (hi >> 12)), (int)((hi << 20) | (lo >> 12))) - (1.0 - 0x1p-53);
 }
 
 __device__ __forceinline__ float u01_from_word(uint32_t w) {
@@ -205,11 +207,9 @@ __device__ __forceinline__ float m_pow(float x, float e) {
   // x >= 0; exp2(e log2 x) with log2(0) = -inf giving 0 for e > 0
   return exp2f(e * __log2f(x));
 }
-__device__ __forceinline__ void m_sincos_2pi(double u, double* s, double* c) {
-  const double th = 2.0 * PI_D * u;
-  *c = cos(th);
-  *s = sin(th);
-}
+__device__ __forceinline__ void m_sincos_2pi(double u, double* s, double* c) { sincos(2.0 * PI_D * u, s, c); }
+__device__ __forceinline__ float m_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double m_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ void m_sincos_2pi(float u, float* s, float* c) {
   sincospif(2.0f * u, s, c);
 }
@@ -821,17 +821,23 @@ __device__ __forceinline__ void collide_window(const Params<T>& p, T* __restrict
         if constexpr (sizeof(T) == 4) post_from_block(wpost, up);
         else draw_post(k, cell, step, p.k0, p.k1, up);
         T et = T(0.25) * g2;
-        if (uinel < p.p_inel) {
-          const T ec = et + ir[pi];
-          ir[pi] = ec * bl_fraction<T, GEN>(p, up[0], k, cell, step, JX_BL);
-          et = ec - ir[pi];
+        // the fractions do not depend on the energies: a lane's first one (of
+        // i, else of j) in one pass for all lanes, a second pass for lanes
+        // with both
+        const bool bi = uinel < p.p_inel, bj = up[1] < p.p_inel;
+        if (bi || bj) {
+          const T f1 = bl_fraction<T, GEN>(p, bi ? up[0] : up[2], k, cell, step, bi ? JX_BL : JX_BL + 2u);
+          const int q1 = bi ? pi : pj;
+          T ec = et + ir[q1];
+          ir[q1] = ec * f1;
+          et = ec - ir[q1];
           cc.inel += 1;
-        }
-        if (up[1] < p.p_inel) {
-          const T ec = et + ir[pj];
-          ir[pj] = ec * bl_fraction<T, GEN>(p, up[2], k, cell, step, JX_BL + 2u);
-          et = ec - ir[pj];
-          cc.inel += 1;
+          if (bi && bj) {
+            ec = et + ir[pj];
+            ir[pj] = ec * bl_fraction<T, GEN>(p, up[2], k, cell, step, JX_BL + 2u);
+            et = ec - ir[pj];
+            cc.inel += 1;
+          }
         }
         const T gn = T(2) * m_sqrt(et);
         T hv[3];
@@ -1000,6 +1006,8 @@ __device__ __forceinline__ T halving_sum17(const T* v, int lane) {
 // pre32 holds the lane's (stg, stc) loaded earlier).  With `flush` the staged
 // sum is folded into the compensated FP64 accumulators (pre: the lane's acc,
 // comp) and the staging pair is cleared.
+// s[1..16] += the sums over this lane's particles (s[0], the count, is n: the
+// caller's)
 template <typename T>
 __device__ __forceinline__ void sample_accumulate(const T* __restrict__ vx, const T* __restrict__ vy,
                                                   const T* __restrict__ vz, const T* __restrict__ ir, int n,
@@ -1007,24 +1015,23 @@ __device__ __forceinline__ void sample_accumulate(const T* __restrict__ vx, cons
   const int lane = threadIdx.x & 31;
   for (int q = lane; q < n; q += 32) {
     const T a = vx[q], b = vy[q], c = vz[q], e = ir[q];
-    const T v2 = a * a + b * b + c * c;
-    s[0] += T(1);
+    const T v2 = m_fma(a, a, m_fma(b, b, c * c));
     s[1] += a;
     s[2] += b;
     s[3] += c;
-    s[4] += a * a;
-    s[5] += b * b;
-    s[6] += c * c;
-    s[7] += a * b;
-    s[8] += a * c;
-    s[9] += b * c;
-    s[10] += a * v2;
-    s[11] += b * v2;
-    s[12] += c * v2;
+    s[4] = m_fma(a, a, s[4]);
+    s[5] = m_fma(b, b, s[5]);
+    s[6] = m_fma(c, c, s[6]);
+    s[7] = m_fma(a, b, s[7]);
+    s[8] = m_fma(a, c, s[8]);
+    s[9] = m_fma(b, c, s[9]);
+    s[10] = m_fma(a, v2, s[10]);
+    s[11] = m_fma(b, v2, s[11]);
+    s[12] = m_fma(c, v2, s[12]);
     s[13] += e;
-    s[14] += e * a;
-    s[15] += e * b;
-    s[16] += e * c;
+    s[14] = m_fma(e, a, s[14]);
+    s[15] = m_fma(e, b, s[15]);
+    s[16] = m_fma(e, c, s[16]);
   }
 }
 
@@ -1061,6 +1068,7 @@ __device__ __forceinline__ void sample_cell_staged(const float* __restrict__ vx,
   float s[NMOM];
 #pragma unroll
   for (int q = 0; q < NMOM; ++q) s[q] = 0.f;
+  if ((threadIdx.x & 31) == 0) s[0] = (float)n;
   sample_accumulate(vx, vy, vz, ir, n, s);
   sample_fold(halving_sum17(s, threadIdx.x & 31), mom, acc, comp, pre, stg, stc, pre32, flush);
 }
@@ -1079,6 +1087,7 @@ __device__ __forceinline__ void sample_cell_f64(const double* __restrict__ vx, c
   double s[NMOM];
 #pragma unroll
   for (int q = 0; q < NMOM; ++q) s[q] = 0.0;
+  if (lane == 0) s[0] = (double)n;
   sample_accumulate(vx, vy, vz, ir, n, s);
   const double v = halving_sum17(s, lane);
   if (mom < 0) return;
@@ -1095,6 +1104,7 @@ __device__ __forceinline__ float sample_chunk(const float* __restrict__ vx, cons
   float s[NMOM];
 #pragma unroll
   for (int q = 0; q < NMOM; ++q) s[q] = 0.f;
+  if ((threadIdx.x & 31) == 0) s[0] = (float)n;
   sample_accumulate(vx, vy, vz, ir, n, s);
   return halving_sum17(s, threadIdx.x & 31);
 }
