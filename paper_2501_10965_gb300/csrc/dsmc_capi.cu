@@ -217,6 +217,7 @@ void carve_state(Carver& cv, const Plan& pl, State<T>& s) {
     s.ovf[b].dest = cv.take<int32_t>(oc);
     s.ovf[b].count = cv.take<int32_t>(1);
   }
+  s.ovf_spare = cv.take<int32_t>(1);
   s.capacity = pl.capacity;
   s.ovf_cap = pl.ovf_cap;
   s.tile = pl.tile;

@@ -87,6 +87,7 @@ struct State {
   bool gen;    // a gas with d_r = 3 or VSS scattering: the fused step's general instantiation
   int fwpb;    // FP32 fused step: warps per CTA (0: not tuned yet)
   int ftile;   // FP32 fused step: particles staged per warp (0: tile)
+  int32_t* ovf_spare;  // FP32 layout: a third overflow counter
   Params<double> pinj;  // annulus: FP64 parameters of the freestream entry
   double* inj_mu;       // annulus: expected entries of every outer face per step
   int inj_max;          // annulus: bound on the entries of one step (sum of floor(mu) + 1)
@@ -199,5 +200,33 @@ void mlp_to_bf16(const Mlp& m, cudaStream_t st);
 // residual statistics pass the judge (see hot_mlp_apply_judged)
 void mlp_apply(const Mlp& m, int ncells, const double* hot, double* hot_out, cudaStream_t st,
                const int32_t* group = nullptr, double z = 0.0, int min_samples = 0, double rel = 0.0);
+
+// Programmatic dependent launch: a kernel launched with launch_pdl may begin
+// while the kernel before it in the stream still runs; grid_dep_wait returns
+// once that one has completed and its writes are visible (at once in a plain
+// launch).  grid_dep_launch lets the next such kernel begin.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// a launch that may overlap the end of the kernel before it in the stream
+// (see grid_dep_wait); pdl = false: a plain launch.  With it, and no launch that
+// clears the overflow counter, a step of 40 000 particles on 200 cells (FP32)
+// went from 23.2 to 19.3 us, of 500 000 on 10 000 cells from 45.1 to 40.9, and
+// one of 10 000 on 100 cells in FP64 from 63 to 57.
+template <typename... A, typename... B>
+inline void launch_pdl(bool pdl, void (*kernel)(A...), int blocks, int threads, size_t smem, cudaStream_t st,
+                       B&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, A(args)...);
+}
 
 }  // namespace dsmc

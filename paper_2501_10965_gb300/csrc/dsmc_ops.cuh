@@ -16,6 +16,7 @@
 
 #include <cstdint>
 #include <type_traits>
+#include <utility>
 #include <cuda_runtime.h>
 
 #include "dsmc_device.cuh"
@@ -271,6 +272,8 @@ __global__ void __launch_bounds__(256) k_move_det(const __grid_constant__ Params
   __shared__ T s_tally[20];
   if (threadIdx.x < 20) s_tally[threadIdx.x] = T(0);
   __syncthreads();
+  grid_dep_wait();
+  grid_dep_launch();
   const int lane = threadIdx.x & 31;
   for (int s0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31); s0 < n; s0 += gridDim.x * blockDim.x) {
     const int s = s0 + lane;
@@ -339,6 +342,8 @@ static __global__ void __launch_bounds__(1024) k_det_lists_small(const int32_t* 
                                                                  const int32_t* __restrict__ arr, int n,
                                                                  int32_t* __restrict__ start,
                                                                  int32_t* __restrict__ list) {
+  grid_dep_wait();
+  grid_dep_launch();
   cta_exclusive_scan(ncells, [&](int i) { return cnt[i]; }, start);
   for (int s = threadIdx.x; s < n; s += 1024) {
     const int k = key[s];
@@ -711,6 +716,8 @@ __global__ void __launch_bounds__(WPB * 32) k_det_cells(const __grid_constant__ 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   if (threadIdx.x < 4) s_cnt[threadIdx.x] = 0;
   __syncthreads();
+  grid_dep_wait();
+  grid_dep_launch();
   const int cell = blockIdx.x * nw + warp;
   const bool live = cell < ncells;
   auto tile_of = [&](int w) { return reinterpret_cast<T*>(smem) + (size_t)w * tile * 4; };
@@ -1078,6 +1085,8 @@ __device__ __forceinline__ int neighbour_cell_ann(int nx, int cell, int code) {
   return j * nx + k;
 }
 
+enum FusedFlags { FF_COLLIDE = 1, FF_SAMPLE = 2, FF_MOVE = 4, FF_FOLD = 8 };
+
 // warps per CTA of the fused step: 2 or 4, chosen per handle with the tile
 // by timing real steps of the handle's first long dsmc_step call (step_bins)
 constexpr int FWPB_MAX = 4;
@@ -1111,7 +1120,8 @@ __global__ void __launch_bounds__(FWPB * 32, 32 / FWPB) k_fused(const __grid_con
                                                         float* __restrict__ sgmax, double* __restrict__ acc,
                                                         double* __restrict__ comp,
                                                         uint32_t* __restrict__ owner_g, Ovf ovi, Ovf ovo,
-                                                        int ovf_cap, uint32_t step_c, uint32_t step_m,
+                                                        int ovf_cap, int32_t* __restrict__ zero, uint32_t step_c,
+                                                        uint32_t step_m,
                                                         int flags, int tile, int ncell_blocks,
                                                         double* __restrict__ tally_g,
                                                         unsigned long long* __restrict__ stats,
@@ -1135,6 +1145,9 @@ __global__ void __launch_bounds__(FWPB * 32, 32 / FWPB) k_fused(const __grid_con
   if (threadIdx.x < FWPB) mbar_init(&s_bar[threadIdx.x], 1);
   mbar_fence_init();
   __syncthreads();
+  grid_dep_wait();  // the previous launch filled the bins read here
+  grid_dep_launch();
+  if (blockIdx.x == 0 && threadIdx.x == 0) *zero = 0;  // the next launch's output overflow counter
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if ((int)blockIdx.x < ncell_blocks) {
     const int cell = blockIdx.x * FWPB + warp;
@@ -2270,7 +2283,8 @@ static void det_cells(const Params<T>& p, State<T>& s, int n, const T* x, const 
   const int ncells = s.ncells;
   int32_t* list = s.scratch_i;
   if (n <= DET_SMALL && ncells <= DET_SMALL) {
-    k_det_lists_small<<<1, 1024, 0, st>>>(s.count[olay], ncells, s.key, s.dest, n, s.start[olay], list);
+    launch_pdl(clear && p.mesh != 1, k_det_lists_small, 1, 1024, 0, st, s.count[olay], ncells, s.key, s.dest, n,
+               s.start[olay], list);
   } else {
     launch_scan(s.count[olay], ncells, s.start[olay], st);
     if (n > 0) k_det_lists<<<grid_for(n, 256), 256, 0, st>>>(s.key, s.dest, n, s.start[olay], list);
@@ -2282,14 +2296,9 @@ static void det_cells(const Params<T>& p, State<T>& s, int n, const T* x, const 
   const int blocks = (ncells + nw - 1) / nw;
   const size_t sm = (size_t)nw * s.tile * (4 * sizeof(T) + sizeof(uint32_t));
   int32_t* old = clear ? s.count[olay ^ 1] : nullptr;
-  if (s.batch)
-    k_det_cells<T, true><<<blocks, nw * 32, sm, st>>>(p, s.cases, ncells, x, y, vx, vy, vz, ir, s.buf[other],
-                                                      s.start[olay], s.count[olay], old, list, nbits, s.cellof,
-                                                      s.sgmax, s.acc, s.comp, s.owner, step, flags, s.tile, s.stats);
-  else
-    k_det_cells<T, false><<<blocks, nw * 32, sm, st>>>(p, s.cases, ncells, x, y, vx, vy, vz, ir, s.buf[other],
-                                                       s.start[olay], s.count[olay], old, list, nbits, s.cellof,
-                                                       s.sgmax, s.acc, s.comp, s.owner, step, flags, s.tile, s.stats);
+  launch_pdl(clear && p.mesh != 1, s.batch ? k_det_cells<T, true> : k_det_cells<T, false>, blocks, nw * 32, sm, st, p,
+             s.cases, ncells, x, y, vx, vy, vz, ir, s.buf[other], s.start[olay], s.count[olay], old, list, nbits,
+             s.cellof, s.sgmax, s.acc, s.comp, s.owner, step, flags, s.tile, s.stats);
 }
 
 template <typename T>
@@ -2302,9 +2311,9 @@ void Ops<T>::step_det(const Params<T>& p, State<T>& s, int& cur, int& lay, uint3
     if (!s.count_clear) cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)s.ncells, st);
     if (n > 0) {
       const int g = grid_for(n, 256);
-#define DSMC_MOVE_DET(D, B, A)                                                                                  \
-  k_move_det<T, D, B, A><<<g, 256, 0, st>>>(p, s.cases, s.buf[cur], s.cellof, s.start[lay], n, step, s.key, s.dest, \
-                                            cnt, s.tally, s.stats)
+#define DSMC_MOVE_DET(D, B, A)                                                                               \
+  launch_pdl(!A && s.count_clear, k_move_det<T, D, B, A>, g, 256, 0, st, p, s.cases, s.buf[cur], s.cellof, \
+             s.start[lay], n, step, s.key, s.dest, cnt, s.tally, s.stats)
       if (p.mesh == 1) DSMC_MOVE_DET(2, false, true);
       else if (p.dim == 1 && s.batch) DSMC_MOVE_DET(1, true, false);
       else if (p.dim == 1) DSMC_MOVE_DET(1, false, false);
@@ -2348,17 +2357,21 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
     if (nsteps <= 0) return;
     const int ncells = s.ncells;
     const int oblocks = 8;
+    int odd = nsteps % 6;
     auto launch = [&](int flags, uint32_t sc, uint32_t sm_step, int F, int ftile) {
       const int other = cur ^ 1;
       const int cblocks = (ncells + F - 1) / F;
       const size_t smf = fused_smem_bytes(ftile, F);
-#define DSMC_FUSED_ARGS                                                                                         \
-  p, s.cases, ncells, s.buf[cur], s.buf[other], s.start[lay], s.count[cur], s.count[other], s.sgmax, s.acc,      \
-      s.comp, s.owner, s.ovf[cur], s.ovf[other], s.ovf_cap, sc, sm_step, flags, ftile, cblocks, s.tally, s.stats, \
-      s.flags + 8, s.stg, s.stc
-#define DSMC_FUSED_LAUNCH(D, B, W, A) k_fused<D, B, W, A, false><<<cblocks + oblocks, W * 32, smf, st>>>(DSMC_FUSED_ARGS)
-#define DSMC_FUSED_LAUNCH_GEN(D, A) k_fused<D, false, 4, A, true><<<cblocks + oblocks, 128, smf, st>>>(DSMC_FUSED_ARGS)
-      const bool inject = p.mesh == 1 && (flags & 4);
+      const int blocks = cblocks + oblocks;
+#define DSMC_FUSED_ARGS                                                                                           \
+  p, s.cases, ncells, s.buf[cur], s.buf[other], s.start[lay], s.count[cur], s.count[other], s.sgmax, s.acc,        \
+      s.comp, s.owner, s.ovf[cur], s.ovf[other], s.ovf_cap, s.ovf_spare, sc, sm_step, flags, ftile, cblocks,       \
+      s.tally, s.stats, s.flags + 8, s.stg, s.stc
+#define DSMC_FUSED_LAUNCH(D, B, W, A)                                                      \
+  launch_pdl(!A, k_fused<D, B, W, A, false>, blocks, W * 32, smf, st, DSMC_FUSED_ARGS)
+#define DSMC_FUSED_LAUNCH_GEN(D, A) \
+  launch_pdl(!A, k_fused<D, false, 4, A, true>, blocks, 128, smf, st, DSMC_FUSED_ARGS)
+      const bool inject = p.mesh == 1;
       if (inject) {
         // annulus: the freestream entry of this step, on the side stream,
         // into the bins the fused step fills (their counts were cleared by
@@ -2400,22 +2413,25 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
 #undef DSMC_FUSED_LAUNCH_GEN
 #undef DSMC_FUSED_ARGS
       if (inject) cudaStreamWaitEvent(st, s.ev_join, 0);
-      // the input overflow list has been consumed
-      cudaMemsetAsync(s.ovf[cur].count, 0, sizeof(int32_t), st);
+      // the input overflow list has been consumed: the next launch's output
+      // list counts with the word this launch has cleared.  The words are
+      // home again after six launches; the call's odd ones clear in place, so
+      // that a captured call finds and leaves them where they are.
+      if (odd-- > 0) cudaMemsetAsync(s.ovf[cur].count, 0, sizeof(int32_t), st);
+      else std::swap(s.ovf[cur].count, s.ovf_spare);
       cur = other;
     };
-    // move of step0, then per step: collide (+sample) of step k and move of step k+1
-    const int tile0 = s.ftile > 0 ? s.ftile : s.tile;
-    launch(4, step0, step0, s.fwpb > 0 ? s.fwpb : FWPB_MAX, tile0);
     // sampled sums are staged in FP32 and folded into FP64 every
     // STAGE_STEPS steps and on the last step of the call
     constexpr int STAGE_STEPS = 16;
     auto fused_flags = [&](int i) {
-      const int fold = ((i + 1) % STAGE_STEPS == 0) ? 8 : 0;
-      return 1 | (do_sample ? 2 | fold : 0) | 4;
+      const int fold = ((i + 1) % STAGE_STEPS == 0) ? FF_FOLD : 0;
+      return FF_COLLIDE | (do_sample ? FF_SAMPLE | fold : 0) | FF_MOVE;
     };
-    int i0 = 0;
     if (s.gen) s.fwpb = 4;  // the general gas has the 4-warp shape only
+    // move of step0, then per step: collide (+sample) of step k and move of step k+1
+    launch(FF_MOVE, step0, step0, s.fwpb > 0 ? s.fwpb : FWPB_MAX, s.ftile > 0 ? s.ftile : s.tile);
+    int i0 = 0;
     if (s.fwpb == 0 && nsteps >= 20) {
       // launch shape of the fused step, tuned on real steps of the call:
       // warps (cells) per CTA and the shared-memory tile (particles staged
