@@ -737,14 +737,18 @@ __device__ __forceinline__ uint32_t ntc_candidates(const Params<T>& p, int n, ui
 // G = 8: four cells side by side, each with its own arguments).  The window
 // then holds up to G candidates; the result does not depend on its size.
 // Every lane of the warp calls it (M = 0 where a group has nothing to do).
+// om: particle q claims word q & om of owner[]; where owner[] has fewer words
+// than particles, two particles that share one only make a candidate wait
+// that could have run.
 template <typename T, bool GEN, int G>
 __device__ __forceinline__ void collide_window(const Params<T>& p, T* __restrict__ vx, T* __restrict__ vy,
                              T* __restrict__ vz, T* __restrict__ ir, int n, uint32_t cell,
-                             uint32_t step, T sgmax, uint32_t M, T* sgmax_ptr, uint32_t* owner, CollCount& cc) {
+                             uint32_t step, T sgmax, uint32_t M, T* sgmax_ptr, uint32_t* owner, CollCount& cc,
+                             uint32_t om = 0xFFFFFFFFu) {
   const int lane = threadIdx.x & 31, gl = lane & (G - 1);
   const unsigned group = (G == 32) ? FULL : (((1u << (G & 31)) - 1u) << (lane & ~(G - 1)));
   if (M != 0u)
-    for (int q = gl; q < n; q += G) owner[q] = OWNER_FREE;
+    for (uint32_t q = gl; q < min((uint32_t)n - 1u, om) + 1u; q += G) owner[q] = OWNER_FREE;
   __syncwarp();
   T obs = T(0);
   uint32_t next = 0;
@@ -788,15 +792,15 @@ __device__ __forceinline__ void collide_window(const Params<T>& p, T* __restrict
     }
     if (__ballot_sync(FULL, has) == 0u) break;
     if (has) {
-      atomicMin(&owner[pi], k);
-      atomicMin(&owner[pj], k);
+      atomicMin(&owner[(uint32_t)pi & om], k);
+      atomicMin(&owner[(uint32_t)pj & om], k);
     }
     __syncwarp();
-    const bool ready = has && owner[pi] == k && owner[pj] == k;
+    const bool ready = has && owner[(uint32_t)pi & om] == k && owner[(uint32_t)pj & om] == k;
     __syncwarp();
     if (has) {
-      owner[pi] = OWNER_FREE;
-      owner[pj] = OWNER_FREE;
+      owner[(uint32_t)pi & om] = OWNER_FREE;
+      owner[(uint32_t)pj & om] = OWNER_FREE;
     }
     __syncwarp();
     if (ready) {

@@ -664,14 +664,8 @@ static __global__ void __launch_bounds__(32) k_inject_bins(const __grid_constant
 
 template <typename T>
 __device__ __forceinline__ void flush_counts(const CollCount& cc, unsigned* s_cnt) {
-  unsigned a = cc.cand, b = cc.coll, c = cc.clip, d = cc.inel;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a += __shfl_xor_sync(FULL, a, o);
-    b += __shfl_xor_sync(FULL, b, o);
-    c += __shfl_xor_sync(FULL, c, o);
-    d += __shfl_xor_sync(FULL, d, o);
-  }
+  const unsigned a = __reduce_add_sync(FULL, cc.cand), b = __reduce_add_sync(FULL, cc.coll);
+  const unsigned c = __reduce_add_sync(FULL, cc.clip), d = __reduce_add_sync(FULL, cc.inel);
   if ((threadIdx.x & 31) == 0) {
     atomicAdd(s_cnt + 0, a);
     atomicAdd(s_cnt + 1, b);
@@ -1107,9 +1101,19 @@ inline size_t fused_smem_bytes(int tile, int fwpb) { return (size_t)fwpb * tile 
 // Move and append: (M1) fly every particle to find its destination and its
 // rank among the cell's particles bound for the same neighbour (shared-memory
 // counters over the 3 x 3 neighbourhood); (M2) one global atomicAdd per
-// destination bin reserves the slots; (M3) fly again (the same counter-based
-// random stream, so the same result) and store.  Counters are flushed by the
-// last warp of the block to finish, so warps never wait for one another.
+// destination bin reserves the slots; (M3) store: a straight flight goes to its
+// reserved slot with no further look at the bin; a particle that reaches a
+// wall or goes far is flown in full (the same counter-based random stream, so
+// the same result), with wall tallies, and takes a slot by itself.  Counters
+// are flushed by the last warp of the block to finish, so warps never wait for
+// one another.
+//
+// Instruction issue (56-65 % of the cycles) and a cell's chain of phases bound
+// it, not HBM.  Cells above the tile, most of a stretched annulus's outer ones,
+// collide in global memory; their owner table is a hash table in the warp's
+// tile (in global memory before).  A step of 20 M particles around the
+// cylinder: 401 us with owners in global memory and every particle's flight
+// repeated in M3, 382 us now; of the 64 1D cases, 99 and 97 us.
 template <int DIM, bool BATCH, int FWPB, bool ANN, bool GEN>
 __global__ void __launch_bounds__(FWPB * 32, 32 / FWPB) k_fused(const __grid_constant__ Params<float> pk,
                                                         Cases<float> cases, int ncells, PBuf<float> in,
@@ -1119,9 +1123,8 @@ __global__ void __launch_bounds__(FWPB * 32, 32 / FWPB) k_fused(const __grid_con
                                                         int32_t* __restrict__ cnt_out,
                                                         float* __restrict__ sgmax, double* __restrict__ acc,
                                                         double* __restrict__ comp,
-                                                        uint32_t* __restrict__ owner_g, Ovf ovi, Ovf ovo,
-                                                        int ovf_cap, int32_t* __restrict__ zero, uint32_t step_c,
-                                                        uint32_t step_m,
+                                                        Ovf ovi, Ovf ovo, int ovf_cap,
+                                                        int32_t* __restrict__ zero, uint32_t step_c, uint32_t step_m,
                                                         int flags, int tile, int ncell_blocks,
                                                         double* __restrict__ tally_g,
                                                         unsigned long long* __restrict__ stats,
@@ -1134,7 +1137,8 @@ __global__ void __launch_bounds__(FWPB * 32, 32 / FWPB) k_fused(const __grid_con
   __shared__ unsigned long long s_hits[2];
   __shared__ unsigned s_done;
   __shared__ unsigned s_out;  // annulus: particles that left
-  __shared__ int s_nb[FWPB][4][12];  // per warp: count, base, bin start, bin capacity
+  __shared__ int s_nb[FWPB][12];     // per warp and destination: particles bound there
+  __shared__ int2 s_slot[FWPB][12];  // ... the first reserved slot in the arrays, slots that fit
   __shared__ __align__(8) uint64_t s_bar[FWPB];
   if (threadIdx.x < 4) s_cnt[threadIdx.x] = 0;
   if (threadIdx.x < 2) s_misc[threadIdx.x] = 0;
@@ -1221,10 +1225,7 @@ __global__ void __launch_bounds__(FWPB * 32, 32 / FWPB) k_fused(const __grid_con
             mtot += sample_chunk(vx, vy, vz, ir, m);
         }
         if (flags & 4) {
-          int* nb_cnt = s_nb[warp][0];
-          int* nb_base = s_nb[warp][1];
-          int* nb_s0 = s_nb[warp][2];
-          int* nb_cap = s_nb[warp][3];
+          int* nb_cnt = s_nb[warp];
           if (lane < 12) nb_cnt[lane] = 0;
           __syncwarp();
           // M1: destinations and ranks; a particle that reaches a wall is
@@ -1249,55 +1250,58 @@ __global__ void __launch_bounds__(FWPB * 32, 32 / FWPB) k_fused(const __grid_con
           // M2: reserve the slots, one atomic per destination bin
           if (lane < 9 && nb_cnt[lane] > 0) {
             const int d = ANN ? neighbour_cell_ann(p.nx, cell, lane) : neighbour_cell(p.nx, cell, lane);
-            nb_base[lane] = atomicAdd(&cnt_out[d], nb_cnt[lane]);
-            const int s0 = start[d];
-            nb_s0[lane] = s0;
-            nb_cap[lane] = start[d + 1] - s0;
+            const int want = nb_cnt[lane];
+            const int b0 = atomicAdd(&cnt_out[d], want);
+            const int bs = start[d], cap = start[d + 1] - bs;
+            s_slot[warp][lane] = make_int2(bs + b0, cap - b0);
+            if (b0 + want > cap - 8) atomicAdd(s_misc + 1, 1u);
           }
           __syncwarp();
-          // M3: fly again (identical result) with wall tallies, and store
+          // M3: store; a particle that reaches a wall or goes far is flown in
+          // full, with wall tallies
           for (int q = lane; q < m; q += 32) {
             float x = px[q], y = (DIM == 2) ? py[q] : 0.f;
             float a = vx[q], b = vy[q], c = vz[q], e = ir[q];
             const uint32_t tag = own[q];
             const int code = (int)(tag >> 24), r = (int)(tag & 0xFFFFFFu);
-            if constexpr (ANN) {
-              if (code < 9) {
-                x = x + a * p.dt;
-                y = y + b * p.dt;
-              } else if (!fly_ann<float, true, GEN>(p, x, y, a, b, c, e, TAG_WALL, (uint32_t)(q0 + q), (uint32_t)lcell, step_m, 0u,
-                                               p.dt, s_tally, &s_hits[0], &s_hits[1])) {
-                atomicAdd(&s_out, 1u);  // left through the outer circle
-                continue;
-              }
-            } else {
-              fly<float, DIM, true, GEN>(p, x, y, a, b, c, e, (uint32_t)(q0 + q), (uint32_t)lcell, step_m, s_tally, &s_hits[0],
-                                    &s_hits[1]);
-            }
-            int d = -1, slot, s0, cap;
+            int d = -1, w;
+            bool fits;
             if (code < 9) {
-              slot = nb_base[code] + r;
-              s0 = nb_s0[code];
-              cap = nb_cap[code];
+              x = x + a * p.dt;
+              if (DIM == 2) y = y + b * p.dt;
+              const int2 sl = s_slot[warp][code];
+              w = sl.x + r;
+              fits = r < sl.y;
             } else {
-              d = ANN ? cell_of_ann<float>(p, x, y) : c0 + cell_of<float, DIM>(p, x, y);
-              if (ANN && d < 0) {
-                atomicAdd(&s_out, 1u);
-                continue;
+              if constexpr (ANN) {
+                if (!fly_ann<float, true, GEN>(p, x, y, a, b, c, e, TAG_WALL, (uint32_t)(q0 + q), (uint32_t)lcell, step_m, 0u,
+                                               p.dt, s_tally, &s_hits[0], &s_hits[1])) {
+                  atomicAdd(&s_out, 1u);  // left through the outer circle
+                  continue;
+                }
+                d = cell_of_ann<float>(p, x, y);
+                if (d < 0) {
+                  atomicAdd(&s_out, 1u);
+                  continue;
+                }
+              } else {
+                fly<float, DIM, true, GEN>(p, x, y, a, b, c, e, (uint32_t)(q0 + q), (uint32_t)lcell, step_m, s_tally, &s_hits[0],
+                                      &s_hits[1]);
+                d = c0 + cell_of<float, DIM>(p, x, y);
               }
-              slot = atomicAdd(&cnt_out[d], 1);
-              s0 = start[d];
-              cap = start[d + 1] - s0;
+              const int slot = atomicAdd(&cnt_out[d], 1);
+              const int bs = start[d], cap = start[d + 1] - bs;
+              w = bs + slot;
+              fits = slot < cap;
+              if (slot >= cap - 8) atomicAdd(s_misc + 1, 1u);
             }
-            if (slot < cap) {
-              const int w = s0 + slot;
+            if (fits) {
               out.x[w] = x;
               if (DIM == 2) out.y[w] = y;
               out.vx[w] = a;
               out.vy[w] = b;
               out.vz[w] = c;
               out.ir[w] = e;
-              if (slot >= cap - 8) atomicAdd(s_misc + 1, 1u);
             } else {
               // reserved but unused slot: give it back (the bin's count ends
               // at its capacity)
@@ -1336,8 +1340,14 @@ __global__ void __launch_bounds__(FWPB * 32, 32 / FWPB) k_fused(const __grid_con
           // and the move chunk by chunk through the tile
           if (flags & 1) {
             CollCount cc{0, 0, 0, 0};
-            collide_cell<float, GEN>(p, in.vx + base, in.vy + base, in.vz + base, in.ir + base, n, (uint32_t)lcell, step_c,
-                                sgmax + cell, owner_g + base, cc);
+            // owners: a hash table over the warp's tile (nothing is staged yet)
+            const float sgm = sgmax[cell];
+            const uint32_t M = ntc_candidates<float>(p, n, (uint32_t)lcell, step_c, sgm);
+            if (M != 0u)
+              collide_window<float, GEN, 32>(p, in.vx + base, in.vy + base, in.vz + base, in.ir + base, n,
+                                             (uint32_t)lcell, step_c, sgm, M, sgmax + cell,
+                                             reinterpret_cast<uint32_t*>(tvx), cc,
+                                             (0x80000000u >> __clz(7 * tile)) - 1u);
             flush_counts<float>(cc, s_cnt);
             fence_proxy_async_global();  // the bulk copies below read these velocities
             __syncwarp();
@@ -2365,8 +2375,8 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
       const int blocks = cblocks + oblocks;
 #define DSMC_FUSED_ARGS                                                                                           \
   p, s.cases, ncells, s.buf[cur], s.buf[other], s.start[lay], s.count[cur], s.count[other], s.sgmax, s.acc,        \
-      s.comp, s.owner, s.ovf[cur], s.ovf[other], s.ovf_cap, s.ovf_spare, sc, sm_step, flags, ftile, cblocks,       \
-      s.tally, s.stats, s.flags + 8, s.stg, s.stc
+      s.comp, s.ovf[cur], s.ovf[other], s.ovf_cap, s.ovf_spare, sc, sm_step, flags, ftile, cblocks, s.tally,       \
+      s.stats, s.flags + 8, s.stg, s.stc
 #define DSMC_FUSED_LAUNCH(D, B, W, A)                                                      \
   launch_pdl(!A, k_fused<D, B, W, A, false>, blocks, W * 32, smf, st, DSMC_FUSED_ARGS)
 #define DSMC_FUSED_LAUNCH_GEN(D, A) \
