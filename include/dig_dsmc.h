@@ -364,13 +364,14 @@ int dsmc_get_volumes(dsmc_handle *h, double *host_out);
  * of a simulated particle (multiply by F = rho V / N for physical units). */
 int dsmc_get_wall_tally(dsmc_handle *h, double *host_out20);
 
-/* Launch shape of the FP32 fused step (host): warps (= cells) per CTA, 2
- * or 4.  A handle times four shapes -- 4 warps with the tile sized from the
- * particles per cell, 2 warps, and 4 warps with the tile 32 particles
- * smaller and larger -- on real steps of its first dsmc_step call of at
- * least 20 steps and keeps the fastest (the first unless another is faster
- * by more than 1 %); 0 before that call and in the FP64-deterministic mode.
- * The paper has no counterpart. */
+/* Launch shape of the FP32 fused step (host): warps per CTA, 2 or 4.  A
+ * handle times four shapes -- 4 warps with the tile sized from the particles
+ * per cell, 2 warps, 4 warps with the tile 32 particles larger, and 4 warps
+ * with the tile 32 smaller or, below 4 864 cells, with all of them on one
+ * cell and a quarter of the tile each -- on real steps of its first dsmc_step
+ * call of at least 20 steps and keeps the fastest (the first unless another
+ * is faster by more than 1 %); 0 before that call and in the
+ * FP64-deterministic mode.  The paper has no counterpart. */
 int dsmc_get_launch_config(dsmc_handle *h, int *host_warps_per_cta);
 
 /* The same launch shape with its tile: particles staged per warp in shared

@@ -1425,6 +1425,12 @@ __global__ void __launch_bounds__(FWPB * 32, 32 / FWPB) k_fused(const __grid_con
   }
 }
 
+}  // namespace dsmc
+
+#include "dsmc_team.cuh"
+
+namespace dsmc {
+
 static __global__ void k_zero_i32(int32_t* a, int n) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) a[i] = 0;
 }
@@ -2368,17 +2374,23 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
     const int ncells = s.ncells;
     const int oblocks = 8;
     int odd = nsteps % 6;
-    auto launch = [&](int flags, uint32_t sc, uint32_t sm_step, int F, int ftile) {
+    // one launch with F warps per CTA; team: a CTA per cell
+    auto launch = [&](int flags, uint32_t sc, uint32_t sm_step, int F, int ftile, bool team) {
       const int other = cur ^ 1;
-      const int cblocks = (ncells + F - 1) / F;
+      const int cblocks = team ? ncells : (ncells + F - 1) / F;
       const size_t smf = fused_smem_bytes(ftile, F);
       const int blocks = cblocks + oblocks;
 #define DSMC_FUSED_ARGS                                                                                           \
   p, s.cases, ncells, s.buf[cur], s.buf[other], s.start[lay], s.count[cur], s.count[other], s.sgmax, s.acc,        \
       s.comp, s.ovf[cur], s.ovf[other], s.ovf_cap, s.ovf_spare, sc, sm_step, flags, ftile, cblocks, s.tally,       \
       s.stats, s.flags + 8, s.stg, s.stc
+#define DSMC_TEAM_ARGS                                                                                            \
+  p, s.cases, ncells, s.buf[cur], s.buf[other], s.start[lay], s.count[cur], s.count[other], s.sgmax, s.acc,        \
+      s.comp, s.ovf[cur], s.ovf[other], s.ovf_cap, s.ovf_spare, sc, sm_step, flags, ftile, cblocks, s.tally,       \
+      s.stats, s.flags + 8, s.stg, s.stc
 #define DSMC_FUSED_LAUNCH(D, B, W, A)                                                      \
   launch_pdl(!A, k_fused<D, B, W, A, false>, blocks, W * 32, smf, st, DSMC_FUSED_ARGS)
+#define DSMC_TEAM_LAUNCH(D, B) launch_pdl(true, k_fused_team<D, B>, blocks, TEAM_WARPS * 32, smf, st, DSMC_TEAM_ARGS)
 #define DSMC_FUSED_LAUNCH_GEN(D, A) \
   launch_pdl(!A, k_fused<D, false, 4, A, true>, blocks, 128, smf, st, DSMC_FUSED_ARGS)
       const bool inject = p.mesh == 1;
@@ -2402,6 +2414,14 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
       } else if (p.mesh == 1) {
         if (F == 2) DSMC_FUSED_LAUNCH(2, false, 2, true);
         else DSMC_FUSED_LAUNCH(2, false, 4, true);
+      } else if (team) {
+        if (p.dim == 1) {
+          if (s.batch) DSMC_TEAM_LAUNCH(1, true);
+          else DSMC_TEAM_LAUNCH(1, false);
+        } else {
+          if (s.batch) DSMC_TEAM_LAUNCH(2, true);
+          else DSMC_TEAM_LAUNCH(2, false);
+        }
       } else if (F == 2) {
         if (p.dim == 1) {
           if (s.batch) DSMC_FUSED_LAUNCH(1, true, 2, false);
@@ -2420,6 +2440,8 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
         }
       }
 #undef DSMC_FUSED_LAUNCH
+#undef DSMC_TEAM_LAUNCH
+#undef DSMC_TEAM_ARGS
 #undef DSMC_FUSED_LAUNCH_GEN
 #undef DSMC_FUSED_ARGS
       if (inject) cudaStreamWaitEvent(st, s.ev_join, 0);
@@ -2440,18 +2462,22 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
     };
     if (s.gen) s.fwpb = 4;  // the general gas has the 4-warp shape only
     // move of step0, then per step: collide (+sample) of step k and move of step k+1
-    launch(FF_MOVE, step0, step0, s.fwpb > 0 ? s.fwpb : FWPB_MAX, s.ftile > 0 ? s.ftile : s.tile);
+    launch(FF_MOVE, step0, step0, s.fwpb > 0 ? s.fwpb : FWPB_MAX, s.ftile > 0 ? s.ftile : s.tile, s.fteam);
     int i0 = 0;
     if (s.fwpb == 0 && nsteps >= 20) {
-      // launch shape of the fused step, tuned on real steps of the call:
-      // warps (cells) per CTA and the shared-memory tile (particles staged
-      // per warp; larger cells go through the chunked path).  Each shape
-      // runs one warm-up step and three timed steps; the first shape (4
+      // launch shape of the fused step, tuned on real steps of the call: warps
+      // per CTA, the shared-memory tile (particles staged per warp; larger
+      // cells go through the tile in chunks) and a warp or a CTA per cell.
+      // Each shape runs one warm-up step and three timed steps; the first (4
       // warps, the tile sized from the particles per cell) is kept unless
-      // another is faster by more than 1 % (the timing's resolution).
+      // another is faster by more than 1 % (the timing's resolution).  A CTA
+      // per cell is tried where the cells do not fill the GPU's warp slots
+      // (152 SMs x 32 warps) in place of the smaller tile.
       const int t0 = s.tile;
       const int tlo = t0 - 32 >= 64 ? t0 - 32 : t0, thi = t0 + 32 <= TILE_MAX_OF<T> ? t0 + 32 : t0;
-      const int shapes[4][2] = {{4, t0}, {2, t0}, {4, tlo}, {4, thi}};
+      const bool few = p.mesh != 1 && ncells < 152 * 32;
+      const int tq = ((t0 + 3) / 4 + 15) & ~15;
+      const int shapes[4][3] = {{4, t0, 0}, {2, t0, 0}, {4, few ? tq : tlo, few ? 1 : 0}, {4, thi, 0}};
       cudaEvent_t ev[8];
       for (auto& e : ev) cudaEventCreate(&e);
       int i = 0;
@@ -2459,7 +2485,7 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
         for (int r = 0; r < 4; ++r, ++i) {
           if (r == 1) cudaEventRecord(ev[2 * k], st);
           const uint32_t sc = step0 + (uint32_t)i;
-          launch(fused_flags(i), sc, sc + 1, shapes[k][0], shapes[k][1]);
+          launch(fused_flags(i), sc, sc + 1, shapes[k][0], shapes[k][1], shapes[k][2] != 0);
         }
         cudaEventRecord(ev[2 * k + 1], st);
       }
@@ -2472,6 +2498,7 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
         if (tk[k] > 0.f && tk[k] < 0.99f * tk[best]) best = k;
       s.fwpb = shapes[best][0];
       s.ftile = shapes[best][1];
+      s.fteam = shapes[best][2] != 0;
       i0 = i;
     }
     const int F = s.fwpb > 0 ? s.fwpb : FWPB_MAX;
@@ -2480,7 +2507,7 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
       const bool last = (i == nsteps - 1);
       const uint32_t sc = step0 + (uint32_t)i;
       if (!last) {
-        launch(fused_flags(i), sc, sc + 1, F, FT);
+        launch(fused_flags(i), sc, sc + 1, F, FT, s.fteam);
       } else {
         const int flags = 1 | (do_sample ? 2 : 0);
         if (s.batch)
@@ -2657,6 +2684,11 @@ void Ops<T>::configure(int tile) {
     cudaFuncSetAttribute(k_collide_sample<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   }
   if constexpr (sizeof(T) == 4) {
+    const int smt = (int)fused_smem_bytes(tile, TEAM_WARPS);
+    cudaFuncSetAttribute(k_fused_team<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smt);
+    cudaFuncSetAttribute(k_fused_team<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smt);
+    cudaFuncSetAttribute(k_fused_team<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smt);
+    cudaFuncSetAttribute(k_fused_team<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smt);
     cudaFuncSetAttribute(k_dig_apply_f32<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smd);
     cudaFuncSetAttribute(k_dig_apply_f32<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smd);
     const int sm4 = (int)fused_smem_bytes(tile, 4), sm2 = (int)fused_smem_bytes(tile, 2);
