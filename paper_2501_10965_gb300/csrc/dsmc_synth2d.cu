@@ -12,9 +12,9 @@
 // every other cell) follows from two solves with B (Sherman-Morrison).
 //
 // Factorisation: per panel of nb columns, one CTA factorises the panel (its
-// rows in registers, k_s2_panel_rot, or in shared memory for taller panels),
-// then one launch applies it to the up to kl + ku trailing columns, up to 8
-// columns per CTA.  Substitution: a cluster of 8 CTAs walks the panels,
+// rows in registers, k_s2_panel_rot, or in shared memory for taller panels);
+// it is applied to the up to kl + ku trailing columns by the other CTAs of the
+// next panel's launch (taller panels: by a launch before it).  Substitution: a cluster of 8 CTAs walks the panels,
 // forward then backward, as a data flow (k_s2_subst_df; with one cluster
 // barrier per panel, k_s2_subst_cl, where its rows do not fit the cluster's
 // shared memory; one CTA, k_s2_subst, where no cluster fits).  The launches
@@ -54,6 +54,8 @@ constexpr int S2_SUB_NT = 512;    // the substitutions
 constexpr int S2_PNL_NT = 512;    // the panel factorisation
 constexpr int S2_NREF = 1;        // refinement sweeps after a fresh factorisation
 constexpr int S2_NREF_REUSE = 3;  // refinement sweeps when an earlier factorisation is reused
+constexpr int S2_ROT_H = 1536;     // tallest panel with its rows in registers
+constexpr int S2_SMS = 152;       // the GPU's SMs
 constexpr int S2_SMEM_CAP = 200 * 1024;
 constexpr int S2_SMAP = 256;  // ints of a panel's row maps (k_s2_sprep, k_s2_spush)
 constexpr size_t S2_DF_SMEM_CAP = 200 * 1024;  // rows of the data-flow substitution per CTA (4 copies of 32 floats a block)
@@ -366,6 +368,91 @@ __device__ __forceinline__ unsigned s2_cand_key(float v, bool cand) {
   return (cand && a == a) ? __float_as_uint(a) + 1u : 0u;
 }
 
+// The interchanges and eliminations of the panel at k0 on up to cbt columns
+// cfirst .. clast, by the CTA (the arithmetic of s2::trail_swaps,
+// trail_l11_step and trail_l21, in their order): the column segments arrive by
+// asynchronous copies (zero outside the band), a thread per column applies the
+// interchanges, a warp per column the unit-lower solve with L11 (lane i
+// holding L11's row i), and a thread per row of L21 (its multipliers in
+// registers) updates that row of every column of the CTA.  No copy of the
+// multipliers in shared memory, so the CTAs stay small and many.
+__device__ __forceinline__ void s2_trail_cols(const s2::Grid& g, const S2Work& w, int k0, int cfirst, int clast,
+                                              int cbt) {
+  __shared__ int spv[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nt = blockDim.x;
+  const int nb = w.nb, ldp = g.kl + nb;
+  const int wd = s2::panel_width(g, nb, k0), H = s2::panel_height(g, wd, k0);
+  const int ncols = clast - cfirst + 1 < cbt ? clast - cfirst + 1 : cbt;
+  if (ncols <= 0) return;
+  float* Cs = reinterpret_cast<float*>(s2_smem);
+  const float* Lk = w.Lp + s2::lp_base(g, nb, k0);
+  for (int e = tid; e < ncols * H; e += nt) {
+    const int cc = e / H, r = e - cc * H, c = cfirst + cc;
+    const bool in = s2::in_band(g, k0 + r, c);
+    s2_cp_async4(Cs + e, w.AB + (in ? s2::band_at(g, k0 + r, c) : 0), in ? 4 : 0);
+  }
+  if (tid < wd) spv[tid] = w.piv[k0 + tid] - k0;
+  s2_cp_async_wait_all();
+  __syncthreads();
+  for (int cc = tid; cc < ncols; cc += nt) {
+    float* a = Cs + (size_t)cc * H;
+    for (int j = 0; j < wd; ++j) {
+      const int p = spv[j];
+      if (p != j) {
+        const float t = a[j];
+        a[j] = a[p];
+        a[p] = t;
+      }
+    }
+  }
+  __syncthreads();
+  {
+    const int i = lane, ic = i < wd ? i : wd - 1;
+    float lr[32];
+#pragma unroll
+    for (int jj = 0; jj < 32; ++jj) {
+      const float l = Lk[(size_t)(jj < wd ? jj : wd - 1) * ldp + ic];
+      lr[jj] = (jj < i && i < wd) ? l : 0.0f;
+    }
+    for (int cc = warp; cc < ncols; cc += (nt >> 5)) {
+      float* a = Cs + (size_t)cc * H;
+      float ai = lane < wd ? a[lane] : 0.0f;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        if (j < wd) {
+          const float aj = __shfl_sync(0xffffffffu, ai, j);
+          if (lane > j && lane < wd) ai -= lr[j] * aj;
+        }
+      }
+      if (lane < wd) a[lane] = ai;
+    }
+  }
+  __syncthreads();
+  for (int r = wd + tid; r < H; r += nt) {
+    float l[32];
+#pragma unroll
+    for (int jj = 0; jj < 32; ++jj) l[jj] = Lk[(size_t)(jj < wd ? jj : wd - 1) * ldp + r];
+    for (int cc = 0; cc < ncols; ++cc) {
+      const float* a = Cs + (size_t)cc * H;
+      float acc = 0.0f;
+#pragma unroll
+      for (int jj = 0; jj < 32; ++jj)
+        if (jj < wd) acc += l[jj] * a[jj];
+      Cs[(size_t)cc * H + r] -= acc;
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < ncols * H; e += nt) {
+    const int cc = e / H, r = e - cc * H, c = cfirst + cc;
+    if (s2::in_band(g, k0 + r, c)) w.AB[s2::band_at(g, k0 + r, c)] = Cs[e];
+  }
+}
+
+__global__ void __launch_bounds__(S2_NT) k_s2_trail(const s2::Grid g, S2Work w, int k0, int cbt) {
+  const int wd = s2::panel_width(g, w.nb, k0);
+  s2_trail_cols(g, w, k0, k0 + wd + blockIdx.x * cbt, s2::trail_last(g, k0, wd), cbt);
+}
+
 // The panel factorisation with the rows in registers.  Thread t holds the
 // rows loaded from positions t + s T (s < RPT, T threads), each as 32
 // columns of a frame that starts at column 4 g in steps 4 g .. 4 g + 3 (the
@@ -380,11 +467,28 @@ __device__ __forceinline__ unsigned s2_cand_key(float v, bool cand) {
 // index) until the end, when they are stored at the rows' final positions.
 // The pivots are chosen as in k_s2_panel (largest magnitude, lowest position
 // among equals), and each entry takes the same operations in the same order.
-template <int RPT>
-__global__ void __launch_bounds__(512) k_s2_panel_rot(const s2::Grid g, S2Work w, int k0) {
+//
+// One launch does the panel at k0 and what is left of the panel before it
+// (kp = k0 - 32; none: kp < 0): CTA 0 applies that one to its own 32 columns
+// as it loads them (interchanges by where a row is read from; the rank-32
+// update row by row in registers), the other CTAs to the columns beyond,
+// cbt each.  So the panels' chain does not wait for the trailing columns.
+// 100 x 100 (1 036 rows): 52 us a panel and 23 us its trailing columns as two
+// launches, 57 us as one.  A column's chain of steps over the warps bounds it
+// (barrier, pivot row, division, update, search), not issue.
+template <int RPT, int TMAX>
+__global__ void __launch_bounds__(TMAX) k_s2_panel_rot(const s2::Grid g, S2Work w, int k0, int kp, int cbt) {
+  grid_dep_wait();
+  grid_dep_launch();
+  if (blockIdx.x > 0) {
+    s2_trail_cols(g, w, kp, k0 + 32 + (blockIdx.x - 1) * cbt, s2::trail_last(g, kp, 32), cbt);
+    return;
+  }
   __shared__ unsigned ckey[2][32];
   __shared__ int cpos[2][32];
   __shared__ __align__(16) float crow[2][32][32];  // per warp: its candidate row (frame of the next step)
+  __shared__ __align__(16) float s_u[32][36];      // U of kp in the panel's columns
+  __shared__ short s_src[S2_ROT_H + 32];  // position before the interchanges of kp of the row at each after them
   const int T = blockDim.x, NS = T * RPT, nw = T >> 5;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int wd = s2::panel_width(g, w.nb, k0), H = s2::panel_height(g, wd, k0);
@@ -392,15 +496,92 @@ __global__ void __launch_bounds__(512) k_s2_panel_rot(const s2::Grid g, S2Work w
   float a[RPT][32];
   int pos[RPT];
   bool act[RPT];
+  // rows of the panel before (frame of kp: this panel's row r is its row r + 32)
+  const int Hp = kp >= 0 ? s2::panel_height(g, 32, kp) : 0;  // at most H + 32
+  if (kp >= 0) {
+    const float* Lk = w.Lp + s2::lp_base(g, 32, kp);
+    const int ldp = g.kl + 32;
+    for (int e = tid; e < 32 * 32; e += T) s2_cp_async4(&crow[1][0][0] + e, Lk + (size_t)(e >> 5) * ldp + (e & 31), 4);
+    for (int j = 0; j < 32; ++j) {
+#pragma unroll
+      for (int s = 0; s < RPT; ++s) {
+        const int q = tid + s * T + 32;
+        s2_cp_async4(Ls + (size_t)j * NS + tid + s * T, Lk + (size_t)j * ldp + (q < Hp ? q : 0), q < Hp ? 4 : 0);
+      }
+    }
+    for (int q = tid; q < Hp; q += T) s_src[q] = (short)q;
+    if (tid < 32) cpos[0][tid] = w.piv[kp + tid] - kp;
+    __syncthreads();
+    if (tid == 0) {
+      for (int j = 0; j < 32; ++j) {
+        const int q = cpos[0][j];
+        const short t = s_src[j];
+        s_src[j] = s_src[q];
+        s_src[q] = t;
+      }
+    }
+    __syncthreads();
+  }
 #pragma unroll
   for (int s = 0; s < RPT; ++s) {
     const int r = tid + s * T;
     pos[s] = r;
     act[s] = r < H;
+    const int row = r + 32 < Hp ? kp + s_src[r + 32] : k0 + r;
 #pragma unroll
     for (int c = 0; c < 32; ++c) {
-      const bool in = r < H && c < wd && s2::in_band(g, k0 + r, k0 + c);
-      a[s][c] = in ? w.AB[s2::band_at(g, k0 + r, k0 + c)] : 0.0f;
+      const bool in = r < H && c < wd && s2::in_band(g, row, k0 + c);
+      a[s][c] = in ? w.AB[s2::band_at(g, row, k0 + c)] : 0.0f;
+    }
+  }
+  if (kp >= 0) {
+    // U of kp in this panel's columns: a warp per column, four at a time
+    s2_cp_async_wait_all();
+    __syncthreads();
+    const int row = kp + s_src[lane];
+    for (int c0 = warp; c0 < 32; c0 += 4 * nw) {
+      float u[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int c = c0 + q * nw;
+        const bool in = c < wd && s2::in_band(g, row, k0 + c);
+        u[q] = in ? w.AB[s2::band_at(g, row, k0 + c)] : 0.0f;
+      }
+#pragma unroll 8
+      for (int j = 0; j < 31; ++j) {
+        const float l = crow[1][j][lane];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float uj = __shfl_sync(0xffffffffu, u[q], j);
+          if (lane > j) u[q] -= l * uj;
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int c = c0 + q * nw;
+        if (c < 32) s_u[lane][c] = u[q];
+      }
+    }
+    __syncthreads();
+    for (int e = tid; e < 32 * 32; e += T) {
+      const int r = e & 31, c = e >> 5;
+      if (c < wd && s2::in_band(g, kp + r, k0 + c)) w.AB[s2::band_at(g, kp + r, k0 + c)] = s_u[r][c];
+    }
+#pragma unroll 2
+    for (int j = 0; j < 32; ++j) {
+      float l[RPT];
+#pragma unroll
+      for (int s = 0; s < RPT; ++s) l[s] = Ls[(size_t)j * NS + tid + s * T];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const float4 v = *reinterpret_cast<const float4*>(&s_u[j][4 * q]);
+        const float uv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+#pragma unroll
+          for (int s = 0; s < RPT; ++s) a[s][4 * q + c] -= l[s] * uv[c];
+        }
+      }
     }
   }
   float pbest = -1.0f;
@@ -424,17 +605,20 @@ __global__ void __launch_bounds__(512) k_s2_panel_rot(const s2::Grid g, S2Work w
     }
     const unsigned kw = __reduce_max_sync(0xffffffffu, key);
     const int pw = __reduce_min_sync(0xffffffffu, key == kw ? bp : INT_MAX);
+    // (one lane: a branch per row it may be, stores of four)
     if (kw != 0u && key == kw && bp == pw) {
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (8 * q + 7 >= fc && 8 * q < lim) {  // chunk q of the frame before the shift
+      for (int s = 0; s < RPT; ++s) {
+        if (s == bs) {
 #pragma unroll
-          for (int c = (8 * q > fc ? 8 * q : fc); c < 8 * q + 8; ++c) {
-            float v = a[0][c];
+          for (int q = 0; q < 4; ++q) {
+            if (8 * q < lim) {  // chunk q of the frame before the shift
 #pragma unroll
-            for (int s = 1; s < RPT; ++s)
-              if (s == bs) v = a[s][c];
-            crow[buf][warp][c - sh] = v;
+              for (int c = 8 * q; c < 8 * q + 8; c += 4)
+                if (c >= sh)
+                  *reinterpret_cast<float4*>(&crow[buf][warp][c - sh]) =
+                      make_float4(a[s][c], a[s][c + 1], a[s][c + 2], a[s][c + 3]);
+            }
           }
         }
       }
@@ -498,11 +682,17 @@ __global__ void __launch_bounds__(512) k_s2_panel_rot(const s2::Grid g, S2Work w
       for (int q = 0; q < 4; ++q) {
         if (8 * q + 7 > jj && 8 * q < live) {
 #pragma unroll
-          for (int c = (8 * q > jj ? 8 * q : jj + 1); c < 8 * q + 8; ++c) {
-            const float pc = prow[c];
+          for (int c4 = 8 * q; c4 < 8 * q + 8; c4 += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(prow + c4);
+            const float pc[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-            for (int s = 0; s < RPT; ++s)
-              if (upd[s]) a[s][c] -= l[s] * pc;
+            for (int c = 0; c < 4; ++c) {
+              if (c4 + c > jj) {
+#pragma unroll
+                for (int s = 0; s < RPT; ++s)
+                  if (upd[s]) a[s][c4 + c] -= l[s] * pc[c];
+              }
+            }
           }
         }
       }
@@ -543,87 +733,6 @@ __global__ void __launch_bounds__(512) k_s2_panel_rot(const s2::Grid g, S2Work w
       const int ps = pos[s], cend = ps < wd ? ps : wd;
       for (int c = 0; c < cend; ++c) w.Lp[base + (size_t)c * ldp + ps] = Ls[(size_t)c * NS + id];
     }
-  }
-}
-
-// The panel's interchanges and eliminations on up to cbt trailing columns per
-// CTA (the arithmetic of s2::trail_swaps, trail_l11_step and trail_l21, in
-// their order): the column segments arrive by asynchronous copies (zero
-// outside the band), a thread per column applies the interchanges, a warp
-// per column the unit-lower solve with L11 (lane i holding L11's row i), and
-// a thread per row of L21 (its multipliers in registers) updates that row of
-// every column of the CTA.  No copy of the multipliers in shared memory, so
-// the CTAs stay small and many.
-__global__ void __launch_bounds__(S2_NT) k_s2_trail(const s2::Grid g, S2Work w, int k0, int cbt) {
-  __shared__ int spv[32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nb = w.nb, ldp = g.kl + nb;
-  const int wd = s2::panel_width(g, nb, k0), H = s2::panel_height(g, wd, k0);
-  const int cfirst = k0 + wd + blockIdx.x * cbt;
-  const int clast = s2::trail_last(g, k0, wd);
-  const int ncols = clast - cfirst + 1 < cbt ? clast - cfirst + 1 : cbt;
-  if (ncols <= 0) return;
-  float* Cs = reinterpret_cast<float*>(s2_smem);
-  const float* Lk = w.Lp + s2::lp_base(g, nb, k0);
-  for (int e = tid; e < ncols * H; e += S2_NT) {
-    const int cc = e / H, r = e - cc * H, c = cfirst + cc;
-    const bool in = s2::in_band(g, k0 + r, c);
-    s2_cp_async4(Cs + e, w.AB + (in ? s2::band_at(g, k0 + r, c) : 0), in ? 4 : 0);
-  }
-  if (tid < wd) spv[tid] = w.piv[k0 + tid] - k0;
-  s2_cp_async_wait_all();
-  __syncthreads();
-  for (int cc = tid; cc < ncols; cc += S2_NT) {
-    float* a = Cs + (size_t)cc * H;
-    for (int j = 0; j < wd; ++j) {
-      const int p = spv[j];
-      if (p != j) {
-        const float t = a[j];
-        a[j] = a[p];
-        a[p] = t;
-      }
-    }
-  }
-  __syncthreads();
-  {
-    const int i = lane, ic = i < wd ? i : wd - 1;
-    float lr[32];
-#pragma unroll
-    for (int jj = 0; jj < 32; ++jj) {
-      const float l = Lk[(size_t)(jj < wd ? jj : wd - 1) * ldp + ic];
-      lr[jj] = (jj < i && i < wd) ? l : 0.0f;
-    }
-    for (int cc = warp; cc < ncols; cc += S2_NT / 32) {
-      float* a = Cs + (size_t)cc * H;
-      float ai = lane < wd ? a[lane] : 0.0f;
-#pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        if (j < wd) {
-          const float aj = __shfl_sync(0xffffffffu, ai, j);
-          if (lane > j && lane < wd) ai -= lr[j] * aj;
-        }
-      }
-      if (lane < wd) a[lane] = ai;
-    }
-  }
-  __syncthreads();
-  for (int r = wd + tid; r < H; r += S2_NT) {
-    float l[32];
-#pragma unroll
-    for (int jj = 0; jj < 32; ++jj) l[jj] = Lk[(size_t)(jj < wd ? jj : wd - 1) * ldp + r];
-    for (int cc = 0; cc < ncols; ++cc) {
-      const float* a = Cs + (size_t)cc * H;
-      float acc = 0.0f;
-#pragma unroll
-      for (int jj = 0; jj < 32; ++jj)
-        if (jj < wd) acc += l[jj] * a[jj];
-      Cs[(size_t)cc * H + r] -= acc;
-    }
-  }
-  __syncthreads();
-  for (int e = tid; e < ncols * H; e += S2_NT) {
-    const int cc = e / H, r = e - cc * H, c = cfirst + cc;
-    if (s2::in_band(g, k0 + r, c)) w.AB[s2::band_at(g, k0 + r, c)] = Cs[e];
   }
 }
 
@@ -2219,13 +2328,13 @@ void s2_smem_limits(size_t panel, size_t trail, size_t subst) {
       set[k] = need[k];
     }
   }
-  // the register-row panels: multipliers of up to 3 x 512 rows
+  // the register-row panels: the multipliers of all rows
   static bool rot_set = false;
   if (!rot_set) {
-    const int cap = (int)(sizeof(float) * 32 * 3 * S2_PNL_NT);
-    cudaFuncSetAttribute(k_s2_panel_rot<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
-    cudaFuncSetAttribute(k_s2_panel_rot<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
-    cudaFuncSetAttribute(k_s2_panel_rot<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
+    const int cap = (int)(sizeof(float) * 32 * S2_ROT_H);
+    const void* rot[4] = {(const void*)k_s2_panel_rot<1, 512>, (const void*)k_s2_panel_rot<1, 1024>,
+                          (const void*)k_s2_panel_rot<2, 640>, (const void*)k_s2_panel_rot<3, 512>};
+    for (const void* f : rot) cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, cap);
     rot_set = true;
   }
 }
@@ -2352,21 +2461,36 @@ int launch_synth2d(const CellParams& cp, const double* fields, const double* hot
     if (refactor) {
       for (int k0 = 0; k0 < g.N; k0 += nb) {
         const int wd = s2::panel_width(g, nb, k0), H = s2::panel_height(g, wd, k0);
-        // rows in registers (up to 3 a thread, 512 threads) where they fit
-        const int rpt = (H + S2_PNL_NT - 1) / S2_PNL_NT;
-        const int tpb = rpt <= 3 ? (H + 32 * rpt - 1) / (32 * rpt) * 32 : 0;
-        const size_t smr = tpb ? sizeof(float) * 32 * (size_t)tpb * rpt : 0;
-        if (nb == 32 && rpt == 1)
-          k_s2_panel_rot<1><<<1, tpb, smr, st>>>(g, w, k0);
-        else if (nb == 32 && rpt == 2)
-          k_s2_panel_rot<2><<<1, tpb, smr, st>>>(g, w, k0);
-        else if (nb == 32 && rpt == 3)
-          k_s2_panel_rot<3><<<1, tpb, smr, st>>>(g, w, k0);
-        else
+        // rows in registers where they fit, the panel before applied in the
+        // same launch.  As few rows a thread as the registers allow: a warp's
+        // chain of a column's steps, not issue, bounds the panel, so more warps
+        // are faster (a whole solve at 60 x 50, 536 rows: 47.6 ms with two rows
+        // a thread, 41.8 with one; 80 x 70, 736 rows: 96.2 and 88.3; 100 x 100,
+        // 1 036 rows: 192 with three, 185 with two)
+        const int rpt = H <= 1024 ? 1 : H <= 1280 ? 2 : H <= S2_ROT_H ? 3 : 0;
+        const int kp = k0 - nb, Hp = k0 > 0 ? s2::panel_height(g, nb, kp) : 0;
+        const int last = k0 > 0 ? s2::trail_last(g, kp, nb) : 0;  // of the panel before
+        if (nb == 32 && rpt > 0) {
+          const int ntrail = k0 > 0 && last >= k0 + wd ? last - (k0 + wd) + 1 : 0;
+          // the trailing columns in one wave of the SMs that the panel leaves
+          int cb = (ntrail + S2_SMS - 2) / (S2_SMS - 1);
+          const int cmax = k0 > 0 ? 32 * S2_ROT_H / Hp : 1;
+          cb = cb < 1 ? 1 : cb < cmax ? cb : cmax;
+          const int grid = 1 + (ntrail + cb - 1) / cb;
+          const int tpb = (H + 32 * rpt - 1) / (32 * rpt) * 32;
+          const size_t smr = sizeof(float) * 32 * (size_t)tpb * rpt;
+          const size_t smt = ntrail ? sizeof(float) * (size_t)cb * Hp : 0;
+          const size_t sm = smr > smt ? smr : smt;
+          auto* kern = rpt == 3   ? k_s2_panel_rot<3, 512>
+                       : rpt == 2 ? k_s2_panel_rot<2, 640>
+                       : tpb > 512 ? k_s2_panel_rot<1, 1024>
+                                   : k_s2_panel_rot<1, 512>;
+          launch_pdl(true, kern, grid, tpb, sm, st, g, w, k0, kp, cb);
+        } else {
+          if (k0 > 0 && last >= k0)
+            k_s2_trail<<<(last - k0 + cbt) / cbt, S2_NT, sizeof(float) * (size_t)cbt * Hp, st>>>(g, w, kp, cbt);
           k_s2_panel<<<1, S2_PNL_NT, sizeof(float) * (size_t)wd * H, st>>>(g, w, k0);
-        const int ntrail = s2::trail_last(g, k0, wd) - (k0 + wd) + 1;
-        if (ntrail > 0)
-          k_s2_trail<<<(ntrail + cbt - 1) / cbt, S2_NT, sizeof(float) * (size_t)cbt * H, st>>>(g, w, k0, cbt);
+        }
       }
       const int nk = (g.N + nb - 1) / nb;
       k_s2_sprep<<<(nk + SP_WPB - 1) / SP_WPB, SP_WPB * 32, 0, st>>>(g, w);
