@@ -14,11 +14,11 @@
 // Factorisation: per panel of nb columns, one CTA factorises the panel (its
 // rows in registers, k_s2_panel_rot, or in shared memory for taller panels);
 // it is applied to the up to kl + ku trailing columns by the other CTAs of the
-// next panel's launch (taller panels: by a launch before it).  Substitution: a cluster of 8 CTAs walks the panels,
-// forward then backward, as a data flow (k_s2_subst_df; with one cluster
-// barrier per panel, k_s2_subst_cl, where its rows do not fit the cluster's
-// shared memory; one CTA, k_s2_subst, where no cluster fits).  The launches
-// on one stream order the factorisation's panels.
+// next panel's launch (taller panels: by a launch before it).  Substitution: a
+// cluster of 8 CTAs walks the panels, forward then backward, as a data flow
+// (k_s2_subst_df; with one cluster barrier per panel, k_s2_subst_cl, where its
+// rows do not fit the cluster's shared memory; one CTA, k_s2_subst, where no
+// cluster fits).  The launches on one stream order the factorisation's panels.
 #include <climits>
 #include <cmath>
 #include <cstdint>
@@ -2181,14 +2181,15 @@ __global__ void k_s2_jvx(const s2::Grid g, S2Work w, int c) {
   w.y1[u] = w.x[u] - e * v;
 }
 
-// s0 = R(y0), s1 = R(y1) (the total-mass row is replaced below)
+// s0 = R(y0), s1 = R(y1) (the total-mass row is replaced below); the second
+// residuals are blockIdx.y = 1's
 __global__ void k_s2_jvres(const s2::Grid g, S2Work w) {
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= g.n) return;
   int i, j;
   s2::cell_of_band(g, b, i, j);
-  s2::cell_residual(g, s2::View{w.y0, -1, 0, 0.0}, i, j, 0.0, w.s0 + s2::NV * b);
-  s2::cell_residual(g, s2::View{w.y1, -1, 0, 0.0}, i, j, 0.0, w.s1 + s2::NV * b);
+  s2::cell_residual(g, s2::View{blockIdx.y ? w.y1 : w.y0, -1, 0, 0.0}, i, j, 0.0,
+                    (blockIdx.y ? w.s1 : w.s0) + s2::NV * b);
 }
 
 // b_c = rhs_c - B v_c
@@ -2437,7 +2438,13 @@ int launch_synth2d(const CellParams& cp, const double* fields, const double* hot
   const size_t sm_subst = sizeof(float) * 2 * ((size_t)g.kl + g.ku + nb);
   s2_smem_limits(sm_panel, sm_trail, sm_subst);
   const int nt = 256;
-  const int cell_grid = (g.n + nt - 1) / nt;
+  // cell residuals: one warp per CTA.  They are long FP64 chains, and CTAs of 8
+  // warps put 1 200 cells on 5 SMs and 10 000 on 40: 123 and 117 us a
+  // residual, 65 and 71 now; the two of a directional difference at 10 000
+  // cells 228 and 84.  (The Jacobian's entries fill the GPU either way, and
+  // CTAs of one warp were slower: 496 and 716 us at 1 200 cells.)
+  const int ntc = 32;
+  const int cell_grid = (g.n + ntc - 1) / ntc;
   const int vec_grid = (g.N + nt - 1) / nt;
   const long long jac_threads = (long long)g.n * s2::NSTENCIL * s2::NV;
   const int jac_grid = (int)((jac_threads + nt - 1) / nt);
@@ -2452,7 +2459,7 @@ int launch_synth2d(const CellParams& cp, const double* fields, const double* hot
   double dm_prev = 0.0;
   for (int it = 0; it < n_m; ++it) {
     k_s2_mass<<<1, S2_NT, 0, st>>>(g, w);
-    k_s2_res<<<cell_grid, nt, 0, st>>>(g, w);
+    k_s2_res<<<cell_grid, ntc, 0, st>>>(g, w);
     // on large grids the Jacobian only where it is factorised: a step that
     // keeps an earlier factorisation refines with directional differences
     const bool jv = !refactor && g.n >= S2_JV_MIN_CELLS;
@@ -2506,7 +2513,7 @@ int launch_synth2d(const CellParams& cp, const double* fields, const double* hot
         k_s2_jveps<<<1, S2_UPD_NT, 0, st>>>(g, w);
         for (int c = 0; c < 2; ++c) {
           k_s2_jvx<<<vec_grid, nt, 0, st>>>(g, w, c);
-          k_s2_jvres<<<cell_grid, nt, 0, st>>>(g, w);
+          k_s2_jvres<<<dim3(cell_grid, 2), ntc, 0, st>>>(g, w);
           k_s2_jvb<<<vec_grid, nt, 0, st>>>(g, w, c);
         }
       }
@@ -2525,7 +2532,7 @@ int launch_synth2d(const CellParams& cp, const double* fields, const double* hot
     dm_prev = sc[S2_DMAX];
   }
   k_s2_mass<<<1, S2_NT, 0, st>>>(g, w);
-  k_s2_res<<<cell_grid, nt, 0, st>>>(g, w);
+  k_s2_res<<<cell_grid, ntc, 0, st>>>(g, w);
   k_s2_final<<<1, S2_NT, 0, st>>>(g, w, out, info);
   cudaMemcpyAsync(sc, w.sc, sizeof(double) * (S2_TOUT + 1), cudaMemcpyDeviceToHost, st);
   cudaError_t e = cudaStreamSynchronize(st);
