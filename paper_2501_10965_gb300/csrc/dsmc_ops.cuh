@@ -1534,6 +1534,9 @@ __device__ __forceinline__ double f2d(float v) {
 __device__ __forceinline__ double to_double(float v) { return f2d(v); }
 __device__ __forceinline__ double to_double(double v) { return v; }
 
+// One warp per cell, 128 particles of it in flight: HBM bounds it (24 B read and
+// 52 B written a particle in FP32).  32 M particles: 612 us one row of 32 at a
+// time, 431 us now (5.6 TB/s).
 template <typename T>
 __global__ void __launch_bounds__(WPB * 32) k_export(PBuf<T> b, const int32_t* __restrict__ start,
                                                      const int32_t* __restrict__ cnt,
@@ -1544,14 +1547,34 @@ __global__ void __launch_bounds__(WPB * 32) k_export(PBuf<T> b, const int32_t* _
   const int cell = blockIdx.x * WPB + warp;
   if (cell >= ncells) return;
   const int si = start[cell], so = ostart[cell], n = cnt[cell];
-  for (int q = lane; q < n; q += 32) {
-    x[so + q] = to_double(b.x[si + q]);
-    y[so + q] = to_double(b.y[si + q]);
-    vx[so + q] = to_double(b.vx[si + q]);
-    vy[so + q] = to_double(b.vy[si + q]);
-    vz[so + q] = to_double(b.vz[si + q]);
-    ir[so + q] = to_double(b.ir[si + q]);
-    cell_out[so + q] = cell;
+  constexpr int U = 4;
+  for (int q0 = lane; q0 < n; q0 += 32 * U) {
+    T v[U][6];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int q = q0 + 32 * u;
+      if (q < n) {
+        v[u][0] = b.x[si + q];
+        v[u][1] = b.y[si + q];
+        v[u][2] = b.vx[si + q];
+        v[u][3] = b.vy[si + q];
+        v[u][4] = b.vz[si + q];
+        v[u][5] = b.ir[si + q];
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int q = q0 + 32 * u;
+      if (q < n) {
+        x[so + q] = to_double(v[u][0]);
+        y[so + q] = to_double(v[u][1]);
+        vx[so + q] = to_double(v[u][2]);
+        vy[so + q] = to_double(v[u][3]);
+        vz[so + q] = to_double(v[u][4]);
+        ir[so + q] = to_double(v[u][5]);
+        cell_out[so + q] = cell;
+      }
+    }
   }
 }
 
@@ -1934,9 +1957,13 @@ __device__ __forceinline__ double exact_scale(uint32_t big) {
 //    floats (both give dig_cell's FP64 values), and only the second moment is
 //    summed in FP64 by every lane, in dig_cell's order;
 //  - the per-cell arithmetic (means, factors) of the CTA's cells is done by
-//    one warp, a lane per cell.
-// 32 M particles (800 x 200 cells, 1D), counts, modification and read-out: 4.28
-// ms with one pass per step of the method and FP64 throughout, 2.50 ms now.
+//    one warp, a lane per cell;
+//  - four CTAs share an SM, so that the others run while one waits at the
+//    barriers around that arithmetic.  The compiler spills 264 bytes a thread
+//    for it, which cost less: 32 M particles (800 x 200 cells, 1D) take 1.81 ms
+//    with two CTAs (no spill), 1.34 with three, 1.14 with four, 1.18 with five.
+// Counts, modification and read-out of the 32 M: 4.28 ms with one pass per step
+// of the method and FP64 throughout, 1.66 ms now.
 constexpr int DIG_FAST = 256;
 struct DigCell {
   int2 s[4];         // exact sums of vx, vy, vz, I_r
@@ -1950,7 +1977,7 @@ struct DigCell {
 };
 
 template <int DIM>
-__global__ void __launch_bounds__(WPB * 32, 2) k_dig_apply_f32(const CellParams* __restrict__ cps,
+__global__ void __launch_bounds__(WPB * 32, 4) k_dig_apply_f32(const CellParams* __restrict__ cps,
                                                             const int32_t* __restrict__ cell_case,
                                                             const int32_t* __restrict__ cell0, int ncells,
                                                             PBuf<float> in, PBuf<float> out,
