@@ -366,7 +366,8 @@ int dsmc_get_wall_tally(dsmc_handle *h, double *host_out20);
 
 /* Launch shape of the FP32 fused step (host): warps per CTA, 2 or 4.  A
  * handle times four shapes -- 4 warps with the tile sized from the particles
- * per cell, 2 warps, 4 warps with the tile 32 particles larger, and 4 warps
+ * per cell, 2 warps, 4 warps with the tile 32 particles larger (on the
+ * annulus: a third smaller), and 4 warps
  * with the tile 32 smaller or, below 4 864 cells, with all of them on one
  * cell and a quarter of the tile each -- on real steps of its first dsmc_step
  * call of at least 20 steps and keeps the fastest (the first unless another

@@ -1114,8 +1114,16 @@ inline size_t fused_smem_bytes(int tile, int fwpb) { return (size_t)fwpb * tile 
 // tile (in global memory before).  A step of 20 M particles around the
 // cylinder: 401 us with owners in global memory and every particle's flight
 // repeated in M3, 382 us now; of the 64 1D cases, 99 and 97 us.
+//
+// Warps per SM the registers are cut for: 32 (64 registers); on the annulus
+// 40 (48 registers, 36 bytes spilled), which the shared memory allows where a
+// smaller tile is chosen: 20 M particles around the cylinder 382 us a step
+// with 32 warps and tile 240, 373 with 40 and 160.  On the boxes 40 was slower
+// (the 64 1D cases 99 and 108 us, 500 000 particles 39.2 and 40.6).
+template <bool ANN, bool GEN>
+constexpr int FUSED_WARPS = (ANN && !GEN) ? 40 : 32;
 template <int DIM, bool BATCH, int FWPB, bool ANN, bool GEN>
-__global__ void __launch_bounds__(FWPB * 32, 32 / FWPB) k_fused(const __grid_constant__ Params<float> pk,
+__global__ void __launch_bounds__(FWPB * 32, FUSED_WARPS<ANN, GEN> / FWPB) k_fused(const __grid_constant__ Params<float> pk,
                                                         Cases<float> cases, int ncells, PBuf<float> in,
                                                         PBuf<float> out,
                                                         const int32_t* __restrict__ start,
@@ -2499,12 +2507,13 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
       // warps, the tile sized from the particles per cell) is kept unless
       // another is faster by more than 1 % (the timing's resolution).  A CTA
       // per cell is tried where the cells do not fill the GPU's warp slots
-      // (152 SMs x 32 warps) in place of the smaller tile.
+      // (152 SMs x 32 warps) in place of the smaller tile; on the annulus two
+      // thirds of the tile, where ten CTAs fit an SM, in place of the larger.
       const int t0 = s.tile;
       const int tlo = t0 - 32 >= 64 ? t0 - 32 : t0, thi = t0 + 32 <= TILE_MAX_OF<T> ? t0 + 32 : t0;
       const bool few = p.mesh != 1 && ncells < 152 * 32;
-      const int tq = ((t0 + 3) / 4 + 15) & ~15;
-      const int shapes[4][3] = {{4, t0, 0}, {2, t0, 0}, {4, few ? tq : tlo, few ? 1 : 0}, {4, thi, 0}};
+      const int tq = ((t0 + 3) / 4 + 15) & ~15, t2 = (2 * t0 / 3 + 15) & ~15;
+      const int shapes[4][3] = {{4, t0, 0}, {2, t0, 0}, {4, few ? tq : tlo, few ? 1 : 0}, {4, p.mesh == 1 ? t2 : thi, 0}};
       cudaEvent_t ev[8];
       for (auto& e : ev) cudaEventCreate(&e);
       int i = 0;
