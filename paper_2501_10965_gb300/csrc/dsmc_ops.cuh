@@ -1113,7 +1113,7 @@ inline size_t fused_smem_bytes(int tile, int fwpb) { return (size_t)fwpb * tile 
 // collide in global memory; their owner table is a hash table in the warp's
 // tile (in global memory before).  A step of 20 M particles around the
 // cylinder: 401 us with owners in global memory and every particle's flight
-// repeated in M3, 382 us now; of the 64 1D cases, 99 and 97 us.
+// repeated in M3, 382 us without; of the 64 1D cases, 99 and 97 us.
 //
 // Warps per SM the registers are cut for: 32 (64 registers); on the annulus
 // 40 (48 registers, 36 bytes spilled), which the shared memory allows where a

@@ -11,10 +11,10 @@ constexpr int TEAM_WARPS = 4;
 // collides, all of them sample and move a share.  With few cells a step takes
 // as long as one cell's chain of phases, whichever SMs idle: 200 cells of 200
 // particles, 20.0 us a step with a warp per cell, 11.8 us with a CTA per cell.
-// Which form a handle takes is
-// timed (step_bins).  Shared memory as k_fused's, the warps' tiles together
-// one tile of TEAM_WARPS * wtile particles; a larger cell collides in global
-// memory (owners: a hash table over the tile) and passes through in chunks.
+// Which form a handle takes is timed (step_bins).  Shared memory as k_fused's,
+// the warps' tiles together one tile of TEAM_WARPS * wtile particles; a larger
+// cell collides in global memory (owners: a hash table over the tile) and
+// passes through in chunks.
 template <int DIM, bool BATCH>
 __global__ void __launch_bounds__(TEAM_WARPS * 32, 8) k_fused_team(
     const __grid_constant__ Params<float> pk, Cases<float> cases, int ncells, PBuf<float> in, PBuf<float> out,
