@@ -1931,23 +1931,31 @@ __device__ __forceinline__ int dig_choice(const CellParams& cp, int q, int n, in
 }
 
 // Exact sum of one value per lane and register slot (v[j] of particle lane +
-// 32 j < n) over the warp: the values scaled by a power of two to 22-bit
-// integers plus 22-bit remainders, added as integers (hi + lo 2^-22, times
-// exact_scale).  big: the bits of the largest magnitude.  Exact down to 2^-44
-// of it, as an FP64 sum is.
+// 32 j < n, n <= 256) over the warp: the values scaled by a power of two to
+// 22-bit integers plus 22-bit remainders, added as integers (hi + lo 2^-22,
+// times exact_scale).  big: the bits of the largest magnitude, below 2^22 so
+// that the scaling loses nothing.  exact is cleared in a lane whose values have
+// bits below the remainder's last one, 2^-43 of the largest's leading bit: the
+// sum is not to be used then.
+// (Adding 1.5 2^23 rounds a float of magnitude up to 2^22 to an integer, which
+// the low bits of the sum's representation hold.)
+constexpr float RND = 12582912.f;
 template <int PER>
-__device__ __forceinline__ int2 exact_sum(const float* v, int n, uint32_t big) {
-  const int lane = threadIdx.x & 31;
+__device__ __forceinline__ int2 exact_sum(const float* v, int n, uint32_t big, bool& exact) {
+  const int lane = threadIdx.x & 31, rnd = __float_as_int(RND);
   // 2^(21 - exponent of the largest): magnitudes below 2^22
   const float up = __uint_as_float((uint32_t)(127 + 21 + 127 - (int)(big >> 23)) << 23);
   int hi = 0, lo = 0;
 #pragma unroll
   for (int j = 0; j < PER; ++j) {
     if (32 * j >= n) break;
-    const float w = (lane + 32 * j < n) ? v[j] * up : 0.f;
-    const int h = __float2int_rn(w);
-    hi += h;
-    lo += __float2int_rn((w - (float)h) * 0x1p22f);
+    const float w = (lane + 32 * j < n) ? __fmul_rn(v[j], up) : 0.f;
+    const float h = __fadd_rn(w, RND);
+    const float r = __fmul_rn(__fsub_rn(w, __fsub_rn(h, RND)), 0x1p22f);  // exact
+    const float l = __fadd_rn(r, RND);
+    hi += __float_as_int(h) - rnd;
+    lo += __float_as_int(l) - rnd;
+    exact = exact && __fsub_rn(l, RND) == r;
   }
   return make_int2(__reduce_add_sync(FULL, hi), __reduce_add_sync(FULL, lo));
 }
@@ -1961,9 +1969,12 @@ __device__ __forceinline__ double exact_scale(uint32_t big) {
 // over memory); others go through dig_cell.  The FP64 pipe (2 lanes per clock
 // and SM, a warp instruction costs 16 cycles for one lane or 32) would bound
 // it, so
-//  - the first moments are exact integer sums, the linear map runs in pairs of
-//    floats (both give dig_cell's FP64 values), and only the second moment is
-//    summed in FP64 by every lane, in dig_cell's order;
+//  - the first moments are integer sums where these are exact (a value's last
+//    bit within 2^-43 of the cell's largest one's first; else FP64 sums about
+//    the first particle, dig_cell's; with thermal values a cell in some
+//    hundreds), the linear map runs in pairs of floats (dig_cell's FP64 values),
+//    and only the second moment is summed in FP64 by every lane, in dig_cell's
+//    order.  So copies of one particle have T_t* = 0 exactly here too;
 //  - the per-cell arithmetic (means, factors) of the CTA's cells is done by
 //    one warp, a lane per cell;
 //  - four CTAs share an SM, so that the others run while one waits at the
@@ -2098,17 +2109,21 @@ __global__ void __launch_bounds__(WPB * 32, 4) k_dig_apply_f32(const CellParams*
 #pragma unroll
     for (int j = 0; j < PER; ++j) probe += (vx[j] + vy[j]) + (vz[j] + ir[j]);  // NaN is not seen by fmaxf
     const uint32_t bv = __reduce_max_sync(FULL, __float_as_uint(big)), bi = __reduce_max_sync(FULL, __float_as_uint(bigi));
-    const bool plain = bv > (64u << 23) && bv < (192u << 23) && bi > (64u << 23) && bi < (192u << 23) &&
-                       __all_sync(FULL, isfinite(probe));
+    // exact_sum's range (up to 2^22), and no bits beyond its last one
+    bool plain = bv > (64u << 23) && bv < (149u << 23) && bi > (64u << 23) && bi < (149u << 23) &&
+                 __all_sync(FULL, isfinite(probe));
     const float rx = __shfl_sync(FULL, vx[0], 0), ry = __shfl_sync(FULL, vy[0], 0), rz = __shfl_sync(FULL, vz[0], 0);
     int2 e[4];
     double sx = 0.0, sy = 0.0, sz = 0.0, si = 0.0;
     if (plain) {
-      e[0] = exact_sum<PER>(vx, np, bv);
-      e[1] = exact_sum<PER>(vy, np, bv);
-      e[2] = exact_sum<PER>(vz, np, bv);
-      e[3] = exact_sum<PER>(ir, np, bi);
-    } else {
+      bool exact = true;
+      e[0] = exact_sum<PER>(vx, np, bv, exact);
+      e[1] = exact_sum<PER>(vy, np, bv, exact);
+      e[2] = exact_sum<PER>(vz, np, bv, exact);
+      e[3] = exact_sum<PER>(ir, np, bi, exact);
+      plain = __all_sync(FULL, exact);
+    }
+    if (!plain) {
       const double dx = f2d(rx), dy = f2d(ry), dz = f2d(rz);
 #pragma unroll
       for (int j = 0; j < PER; ++j)
@@ -2155,7 +2170,8 @@ __global__ void __launch_bounds__(WPB * 32, 4) k_dig_apply_f32(const CellParams*
     const double dn = (double)c.np;
     const double r[3] = {f2d(c.rx), f2d(c.ry), f2d(c.rz)};
     if (c.bv) {
-      // the sums about the first particle: exact, like the sums themselves
+      // the sums about the first particle: exact, as every term is a multiple of
+      // the sums' last bit and the result takes at most 53
       const double kv = exact_scale(c.bv), ki = exact_scale(c.bi);
       for (int q = 0; q < 3; ++q)
         c.sums[q] = __fma_rn(-dn, r[q], __fma_rn((double)c.s[q].y, 0x1p-22, (double)c.s[q].x) * kv);
