@@ -205,7 +205,9 @@ void mlp_apply(const Mlp& m, int ncells, const double* hot, double* hot_out, cud
 // Programmatic dependent launch: a kernel launched with launch_pdl may begin
 // while the kernel before it in the stream still runs; grid_dep_wait returns
 // once that one has completed and its writes are visible (at once in a plain
-// launch).  grid_dep_launch lets the next such kernel begin.
+// launch).  grid_dep_launch lets the next such kernel begin.  Such a kernel's
+// pointers are not __restrict__: the qualifier would promise that nothing else
+// writes the memory while the kernel runs, and a load could move above the wait.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -263,12 +263,12 @@ __device__ __forceinline__ int32_t cell_arrival(int32_t* __restrict__ cnt, int k
 // number in it, cnt = the new occupancies (zero before)
 template <typename T, int DIM, bool BATCH, bool ANN>
 __global__ void __launch_bounds__(256) k_move_det(const __grid_constant__ Params<T> pk, Cases<T> cases, PBuf<T> b,
-                                                  const int32_t* __restrict__ cellof,
-                                                  const int32_t* __restrict__ start, int n,
-                                                  uint32_t step, int32_t* __restrict__ key,
-                                                  int32_t* __restrict__ arr, int32_t* __restrict__ cnt,
-                                                  double* __restrict__ tally_g,
-                                                  unsigned long long* __restrict__ stats) {
+                                                  const int32_t* cellof,
+                                                  const int32_t* start, int n,
+                                                  uint32_t step, int32_t* key,
+                                                  int32_t* arr, int32_t* cnt,
+                                                  double* tally_g,
+                                                  unsigned long long* stats) {
   __shared__ T s_tally[20];
   if (threadIdx.x < 20) s_tally[threadIdx.x] = T(0);
   __syncthreads();
@@ -327,28 +327,34 @@ static __global__ void k_arrivals(const int32_t* __restrict__ key, int n, int32_
   }
 }
 
-// the lists of source slots, in order of arrival
-static __global__ void k_det_lists(const int32_t* __restrict__ key, const int32_t* __restrict__ arr, int n,
-                                   const int32_t* __restrict__ start, int32_t* __restrict__ list) {
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
+// the lists of source slots, in order of arrival: slots s0, s0 + stride, ...
+// (__restrict__ here, not on the parameters of a kernel that overlaps the launch
+// before it: it holds only within this function, behind the kernel's wait, and
+// lets one slot's loads pass another's store)
+__device__ __forceinline__ void list_slots(const int32_t* __restrict__ key, const int32_t* __restrict__ arr, int s0,
+                                           int stride, int n, const int32_t* __restrict__ start,
+                                           int32_t* __restrict__ list) {
+  for (int s = s0; s < n; s += stride) {
     const int k = key[s];
     if (k >= 0) list[start[k] + arr[s]] = s;
   }
 }
 
+static __global__ void k_det_lists(const int32_t* __restrict__ key, const int32_t* __restrict__ arr, int n,
+                                   const int32_t* __restrict__ start, int32_t* __restrict__ list) {
+  list_slots(key, arr, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, n, start, list);
+}
+
 // scan and lists in one CTA, for few particles and cells (one launch less)
-static __global__ void __launch_bounds__(1024) k_det_lists_small(const int32_t* __restrict__ cnt, int ncells,
-                                                                 const int32_t* __restrict__ key,
-                                                                 const int32_t* __restrict__ arr, int n,
-                                                                 int32_t* __restrict__ start,
-                                                                 int32_t* __restrict__ list) {
+static __global__ void __launch_bounds__(1024) k_det_lists_small(const int32_t* cnt, int ncells,
+                                                                 const int32_t* key,
+                                                                 const int32_t* arr, int n,
+                                                                 int32_t* start,
+                                                                 int32_t* list) {
   grid_dep_wait();
   grid_dep_launch();
   cta_exclusive_scan(ncells, [&](int i) { return cnt[i]; }, start);
-  for (int s = threadIdx.x; s < n; s += 1024) {
-    const int k = key[s];
-    if (k >= 0) list[start[k] + arr[s]] = s;
-  }
+  list_slots(key, arr, threadIdx.x, 1024, n, start, list);
 }
 
 // Ascending order of a cell's list that does not fit the tile: one warp,
@@ -674,6 +680,27 @@ __device__ __forceinline__ void flush_counts(const CollCount& cc, unsigned* s_cn
   }
 }
 
+// particles order[0 .. n) of the input arrays to the cell's places (__restrict__:
+// see list_slots)
+template <typename T>
+__device__ __forceinline__ void gather_cell(const int32_t* __restrict__ order, int n, const T* __restrict__ ix,
+                                            const T* __restrict__ iy, const T* __restrict__ ivx,
+                                            const T* __restrict__ ivy, const T* __restrict__ ivz,
+                                            const T* __restrict__ iir, T* __restrict__ x, T* __restrict__ y,
+                                            T* __restrict__ vx, T* __restrict__ vy, T* __restrict__ vz,
+                                            T* __restrict__ ir, int32_t* __restrict__ cellof, int cell) {
+  for (int q = threadIdx.x & 31; q < n; q += 32) {
+    const int s = order[q];
+    x[q] = ix[s];
+    y[q] = iy[s];
+    vx[q] = ivx[s];
+    vy[q] = ivy[s];
+    vz[q] = ivz[s];
+    ir[q] = iir[s];
+    cellof[q] = cell;
+  }
+}
+
 // FP64 layout, one warp per cell: order the cell's list of source slots,
 // gather its particles (positions straight to the output, velocities and
 // energies to shared memory; cells above `tile` particles work in the output
@@ -691,18 +718,18 @@ __device__ __forceinline__ void flush_counts(const CollCount& cc, unsigned* s_cn
 constexpr uint32_t GROUP_MAX_M = 24u;
 template <typename T, bool BATCH>
 __global__ void __launch_bounds__(WPB * 32) k_det_cells(const __grid_constant__ Params<T> pk, Cases<T> cases,
-                                                        int ncells, const T* __restrict__ ix,
-                                                        const T* __restrict__ iy, const T* __restrict__ ivx,
-                                                        const T* __restrict__ ivy, const T* __restrict__ ivz,
-                                                        const T* __restrict__ iir, PBuf<T> b,
-                                                        const int32_t* __restrict__ start,
-                                                        const int32_t* __restrict__ count,
-                                                        int32_t* __restrict__ cnt_old, int32_t* __restrict__ list,
-                                                        int nbits, int32_t* __restrict__ cellof,
-                                                        T* __restrict__ sgmax, double* __restrict__ acc,
-                                                        double* __restrict__ comp, uint32_t* __restrict__ owner_g,
+                                                        int ncells, const T* ix,
+                                                        const T* iy, const T* ivx,
+                                                        const T* ivy, const T* ivz,
+                                                        const T* iir, PBuf<T> b,
+                                                        const int32_t* start,
+                                                        const int32_t* count,
+                                                        int32_t* cnt_old, int32_t* list,
+                                                        int nbits, int32_t* cellof,
+                                                        T* sgmax, double* acc,
+                                                        double* comp, uint32_t* owner_g,
                                                         uint32_t step, int flags, int tile,
-                                                        unsigned long long* __restrict__ stats) {
+                                                        unsigned long long* stats) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned s_cnt[4];
   __shared__ uint32_t s_m[WPB];
@@ -730,6 +757,7 @@ __global__ void __launch_bounds__(WPB * 32) k_det_cells(const __grid_constant__ 
   if (live) {
     base = start[cell];
     n = count[cell];
+    if (flags & 1) sg = sgmax[cell];
     if (lane == 0 && cnt_old) cnt_old[cell] = 0;
     staged = n <= tile;
     const int32_t* order;
@@ -770,22 +798,9 @@ __global__ void __launch_bounds__(WPB * 32) k_det_cells(const __grid_constant__ 
       order = sort_list_global(list + base, reinterpret_cast<int32_t*>(owner_g) + base, n, nbits,
                                reinterpret_cast<int32_t*>(tile_of(warp)));
     }
-    for (int q = lane; q < n; q += 32) {
-      const int s = order[q];
-      const T x = ix[s], y = iy[s], a = ivx[s], bb = ivy[s], c = ivz[s], e = iir[s];
-      b.x[base + q] = x;
-      b.y[base + q] = y;
-      vx[q] = a;
-      vy[q] = bb;
-      vz[q] = c;
-      ir[q] = e;
-      cellof[base + q] = cell;
-    }
+    gather_cell<T>(order, n, ix, iy, ivx, ivy, ivz, iir, b.x + base, b.y + base, vx, vy, vz, ir, cellof + base, cell);
     __syncwarp();
-    if (flags & 1) {
-      sg = sgmax[cell];
-      M = ntc_candidates<T>(p, n, (uint32_t)lcell, step, sg);
-    }
+    if (flags & 1) M = ntc_candidates<T>(p, n, (uint32_t)lcell, step, sg);
   }
   if (flags & 1) {
     CollCount cc{0, 0, 0, 0};
@@ -1126,18 +1141,18 @@ template <int DIM, bool BATCH, int FWPB, bool ANN, bool GEN>
 __global__ void __launch_bounds__(FWPB * 32, FUSED_WARPS<ANN, GEN> / FWPB) k_fused(const __grid_constant__ Params<float> pk,
                                                         Cases<float> cases, int ncells, PBuf<float> in,
                                                         PBuf<float> out,
-                                                        const int32_t* __restrict__ start,
-                                                        int32_t* __restrict__ cnt_in,
-                                                        int32_t* __restrict__ cnt_out,
-                                                        float* __restrict__ sgmax, double* __restrict__ acc,
-                                                        double* __restrict__ comp,
+                                                        const int32_t* start,
+                                                        int32_t* cnt_in,
+                                                        int32_t* cnt_out,
+                                                        float* sgmax, double* acc,
+                                                        double* comp,
                                                         Ovf ovi, Ovf ovo, int ovf_cap,
-                                                        int32_t* __restrict__ zero, uint32_t step_c, uint32_t step_m,
+                                                        int32_t* zero, uint32_t step_c, uint32_t step_m,
                                                         int flags, int tile, int ncell_blocks,
-                                                        double* __restrict__ tally_g,
-                                                        unsigned long long* __restrict__ stats,
-                                                        int32_t* __restrict__ errflag, float* __restrict__ stg,
-                                                        float* __restrict__ stc) {
+                                                        double* tally_g,
+                                                        unsigned long long* stats,
+                                                        int32_t* errflag, float* stg,
+                                                        float* stc) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned s_cnt[4];
   __shared__ unsigned s_misc[2];

@@ -18,11 +18,11 @@ constexpr int TEAM_WARPS = 4;
 template <int DIM, bool BATCH>
 __global__ void __launch_bounds__(TEAM_WARPS * 32, 8) k_fused_team(
     const __grid_constant__ Params<float> pk, Cases<float> cases, int ncells, PBuf<float> in, PBuf<float> out,
-    const int32_t* __restrict__ start, int32_t* __restrict__ cnt_in, int32_t* __restrict__ cnt_out,
-    float* __restrict__ sgmax, double* __restrict__ acc, double* __restrict__ comp, Ovf ovi, Ovf ovo, int ovf_cap,
-    int32_t* __restrict__ zero, uint32_t step_c, uint32_t step_m, int flags, int wtile, int ncell_blocks,
-    double* __restrict__ tally_g, unsigned long long* __restrict__ stats, int32_t* __restrict__ errflag,
-    float* __restrict__ stg, float* __restrict__ stc) {
+    const int32_t* start, int32_t* cnt_in, int32_t* cnt_out,
+    float* sgmax, double* acc, double* comp, Ovf ovi, Ovf ovo, int ovf_cap,
+    int32_t* zero, uint32_t step_c, uint32_t step_m, int flags, int wtile, int ncell_blocks,
+    double* tally_g, unsigned long long* stats, int32_t* errflag,
+    float* stg, float* stc) {
   constexpr int NT = TEAM_WARPS * 32;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned s_cnt[4];
