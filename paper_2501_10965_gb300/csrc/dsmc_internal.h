@@ -64,7 +64,7 @@ struct State {
   double slack;    // FP32 bin capacity = slack * count + 32
   PBuf<T> buf[2];  // particle buffers; buf[cur] holds the state
   int32_t* start[2];  // layout: bin starts (ncells + 1) ...
-  int32_t* count[2];  // ... and occupancies (ncells)
+  int32_t* count[2];  // ... and occupancies (ncells); those not in use are zero
   int32_t* cellof;    // FP64 compact layout: cell of each slot
   int32_t* key;       // scratch: new cell per slot
   int32_t* dest;      // scratch: destination slot
@@ -97,7 +97,6 @@ struct State {
   // atomics); fork after the previous launch, join before the next
   cudaStream_t side;
   cudaEvent_t ev_fork, ev_join;
-  bool count_clear;  // FP64 layout: the occupancies of the layout not in use are zero
   bool lost;  // FP64 annulus: freestream entries did not fit the workspace
 };
 

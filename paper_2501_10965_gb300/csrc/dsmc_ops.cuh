@@ -758,7 +758,7 @@ __global__ void __launch_bounds__(WPB * 32) k_det_cells(const __grid_constant__ 
     base = start[cell];
     n = count[cell];
     if (flags & 1) sg = sgmax[cell];
-    if (lane == 0 && cnt_old) cnt_old[cell] = 0;
+    if (lane == 0) cnt_old[cell] = 0;
     staged = n <= tile;
     const int32_t* order;
     if (staged) {
@@ -2356,16 +2356,17 @@ constexpr int DET_SMALL = 16384;
 
 // FP64 layout: particles with cells `key` and arrival numbers `arr` (n slots
 // of the six input arrays, occupancies s.count[olay]) into buffer `other`,
-// layout olay; then flags as k_det_cells.  clear: the occupancies of the
-// layout left behind are cleared (they are not read again).
+// layout olay; then flags as k_det_cells.  The occupancies of the layout left
+// behind are cleared: outside a call those of the layout not in use are always
+// zero, so that a step counts into them without a look at the host's state (a
+// captured step too).
 template <typename T>
 static void det_cells(const Params<T>& p, State<T>& s, int n, const T* x, const T* y, const T* vx, const T* vy,
-                      const T* vz, const T* ir, int other, int olay, uint32_t step, int flags, bool clear,
-                      cudaStream_t st) {
+                      const T* vz, const T* ir, int other, int olay, uint32_t step, int flags, cudaStream_t st) {
   const int ncells = s.ncells;
   int32_t* list = s.scratch_i;
   if (n <= DET_SMALL && ncells <= DET_SMALL) {
-    launch_pdl(clear && p.mesh != 1, k_det_lists_small, 1, 1024, 0, st, s.count[olay], ncells, s.key, s.dest, n,
+    launch_pdl(p.mesh != 1, k_det_lists_small, 1, 1024, 0, st, s.count[olay], ncells, s.key, s.dest, n,
                s.start[olay], list);
   } else {
     launch_scan(s.count[olay], ncells, s.start[olay], st);
@@ -2377,10 +2378,9 @@ static void det_cells(const Params<T>& p, State<T>& s, int n, const T* x, const 
   const int nw = ncells <= 2 * 152 ? 1 : WPB;
   const int blocks = (ncells + nw - 1) / nw;
   const size_t sm = (size_t)nw * s.tile * (4 * sizeof(T) + sizeof(uint32_t));
-  int32_t* old = clear ? s.count[olay ^ 1] : nullptr;
-  launch_pdl(clear && p.mesh != 1, s.batch ? k_det_cells<T, true> : k_det_cells<T, false>, blocks, nw * 32, sm, st, p,
-             s.cases, ncells, x, y, vx, vy, vz, ir, s.buf[other], s.start[olay], s.count[olay], old, list, nbits,
-             s.cellof, s.sgmax, s.acc, s.comp, s.owner, step, flags, s.tile, s.stats);
+  launch_pdl(p.mesh != 1, s.batch ? k_det_cells<T, true> : k_det_cells<T, false>, blocks, nw * 32, sm, st, p,
+             s.cases, ncells, x, y, vx, vy, vz, ir, s.buf[other], s.start[olay], s.count[olay], s.count[olay ^ 1], list,
+             nbits, s.cellof, s.sgmax, s.acc, s.comp, s.owner, step, flags, s.tile, s.stats);
 }
 
 template <typename T>
@@ -2390,11 +2390,10 @@ void Ops<T>::step_det(const Params<T>& p, State<T>& s, int& cur, int& lay, uint3
     const int n = s.nparticles;
     const int other = cur ^ 1, olay = lay ^ 1;
     int32_t* cnt = s.count[olay];
-    if (!s.count_clear) cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)s.ncells, st);
     if (n > 0) {
       const int g = grid_for(n, 256);
 #define DSMC_MOVE_DET(D, B, A)                                                                               \
-  launch_pdl(!A && s.count_clear, k_move_det<T, D, B, A>, g, 256, 0, st, p, s.cases, s.buf[cur], s.cellof, \
+  launch_pdl(!A, k_move_det<T, D, B, A>, g, 256, 0, st, p, s.cases, s.buf[cur], s.cellof, \
              s.start[lay], n, step, s.key, s.dest, cnt, s.tally, s.stats)
       if (p.mesh == 1) DSMC_MOVE_DET(2, false, true);
       else if (p.dim == 1 && s.batch) DSMC_MOVE_DET(1, true, false);
@@ -2417,8 +2416,7 @@ void Ops<T>::step_det(const Params<T>& p, State<T>& s, int& cur, int& lay, uint3
       if (tot > s.capacity) s.lost = true;  // entries beyond the workspace were not written
     }
     const PBuf<T>& a = s.buf[cur];
-    det_cells<T>(p, s, ntot, a.x, a.y, a.vx, a.vy, a.vz, a.ir, other, olay, step, 1 | (do_sample ? 2 : 0), true, st);
-    s.count_clear = true;
+    det_cells<T>(p, s, ntot, a.x, a.y, a.vx, a.vy, a.vz, a.ir, other, olay, step, 1 | (do_sample ? 2 : 0), st);
     cur = other;
     lay = olay;
     if (p.mesh == 1) {
@@ -2652,10 +2650,8 @@ void Ops<T>::import_particles(const Params<T>& p, State<T>& s, int& cur, int& la
   if (det) {
     if constexpr (sizeof(T) == 8) {
       // sorted by cell into the other buffer, in the given order within a cell
-      cudaMemsetAsync(s.count[olay], 0, sizeof(int32_t) * (size_t)s.ncells, st);
       if (n > 0) k_arrivals<<<grid_for(n, 256), 256, 0, st>>>(s.key, (int)n, s.count[olay], s.dest);
-      det_cells<T>(p, s, (int)n, x, yy, vx, vy, vz, ir, other, olay, 0u, 0, false, st);
-      s.count_clear = false;
+      det_cells<T>(p, s, (int)n, x, yy, vx, vy, vz, ir, other, olay, 0u, 0, st);
     }
     cur = other;
     lay = olay;
@@ -2720,8 +2716,8 @@ void Ops<T>::dig_apply(const CellParams& cp0, State<T>& s, int ncells, int& cur,
     else k_dig_apply_f64<2><<<blocks, WPB * 32, sm, st>>>(DSMC_DIG_ARGS, s.cellof, s.tile);
   }
 #undef DSMC_DIG_ARGS
-  if (det) s.count_clear = false;
-  else k_zero_i32<<<grid_for(ncells, 256), 256, 0, st>>>(s.count[cur], ncells);
+  // the occupancies left behind are cleared: the next step appends to them
+  k_zero_i32<<<grid_for(ncells, 256), 256, 0, st>>>(s.count[cin], ncells);
   cur = other;
   lay = olay;
 }
