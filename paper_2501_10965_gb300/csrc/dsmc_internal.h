@@ -88,7 +88,7 @@ struct State {
   int fwpb;    // FP32 fused step: warps per CTA (0: not tuned yet)
   int ftile;   // FP32 fused step: particles staged per warp (0: tile)
   bool fteam;  // FP32 fused step: a CTA per cell (dsmc_team.cuh)
-  int32_t* ovf_spare;  // FP32 layout: a third overflow counter
+  int32_t* ovf_spare;  // FP32 layout: a third overflow counter; the three words rotate, a launch a turn
   Params<double> pinj;  // annulus: FP64 parameters of the freestream entry
   double* inj_mu;       // annulus: expected entries of every outer face per step
   int inj_max;          // annulus: bound on the entries of one step (sum of floor(mu) + 1)

@@ -2437,7 +2437,6 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
     if (nsteps <= 0) return;
     const int ncells = s.ncells;
     const int oblocks = 8;
-    int odd = nsteps % 6;
     // one launch with F warps per CTA; team: a CTA per cell
     auto launch = [&](int flags, uint32_t sc, uint32_t sm_step, int F, int ftile, bool team) {
       const int other = cur ^ 1;
@@ -2510,11 +2509,9 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
 #undef DSMC_FUSED_ARGS
       if (inject) cudaStreamWaitEvent(st, s.ev_join, 0);
       // the input overflow list has been consumed: the next launch's output
-      // list counts with the word this launch has cleared.  The words are
-      // home again after six launches; the call's odd ones clear in place, so
-      // that a captured call finds and leaves them where they are.
-      if (odd-- > 0) cudaMemsetAsync(s.ovf[cur].count, 0, sizeof(int32_t), st);
-      else std::swap(s.ovf[cur].count, s.ovf_spare);
+      // list counts with the word that this launch has cleared (no clear between
+      // launches, so that all of a call's overlap alike, the timed ones too)
+      std::swap(s.ovf[cur].count, s.ovf_spare);
       cur = other;
     };
     // sampled sums are staged in FP32 and folded into FP64 every
