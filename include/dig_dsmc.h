@@ -365,19 +365,19 @@ int dsmc_get_volumes(dsmc_handle *h, double *host_out);
 int dsmc_get_wall_tally(dsmc_handle *h, double *host_out20);
 
 /* Launch shape of the FP32 fused step (host): warps per CTA, 2 or 4.  A
- * handle times four shapes -- 4 warps with the tile sized from the particles
- * per cell, 2 warps, 4 warps with the tile 32 particles larger (on the
- * annulus: a third smaller), and 4 warps
- * with the tile 32 smaller or, below 4 864 cells, with all of them on one
- * cell and a quarter of the tile each -- on real steps of its first dsmc_step
- * call of at least 20 steps and keeps the fastest (the first unless another
- * is faster by more than 1 %); 0 before that call and in the
- * FP64-deterministic mode.  The paper has no counterpart. */
+ * handle times four shapes on real steps of its first dsmc_step call of at
+ * least 20 steps and keeps the fastest (the first unless another is faster by
+ * more than 1 %): 4 warps, a cell each, with the tile sized from the particles
+ * per cell; 2 warps; 4 warps with the tile 32 particles smaller, or below
+ * 4 864 cells all 4 on one cell with about that tile together; 4 warps with the
+ * tile 32 larger, on the annulus a third smaller.  0 before that call and in
+ * the FP64-deterministic mode.  The paper has no counterpart. */
 int dsmc_get_launch_config(dsmc_handle *h, int *host_warps_per_cta);
 
-/* The same launch shape with its tile: particles staged per warp in shared
- * memory (cells above it take the chunked path); 0, 0 before the tuning
- * call and in the FP64-deterministic mode. */
+/* The same launch shape with its tile: particles of a cell staged in shared
+ * memory (cells above it take the chunked path), by a warp or, where the shape
+ * is a CTA per cell, by the CTA; 0, 0 before the tuning call and in the
+ * FP64-deterministic mode. */
 int dsmc_get_launch_shape(dsmc_handle *h, int *host_warps_per_cta, int *host_tile);
 
 /* Derived constants (host, 8 entries): dx, dy, cell volume V, particle weight

@@ -1171,7 +1171,9 @@ int dsmc_get_constants(dsmc_handle* h, double* out8) {
 int dsmc_get_launch_shape(dsmc_handle* h, int* host_warps_per_cta, int* host_tile) {
   if (!h || !host_warps_per_cta || !host_tile) return set_err(h, DSMC_ERR_ARG, "bad arguments");
   *host_warps_per_cta = h->det ? 0 : h->sf.fwpb;
-  *host_tile = (h->det || h->sf.fwpb == 0) ? 0 : (h->sf.ftile > 0 ? h->sf.ftile : h->sf.tile);
+  // with a CTA per cell its warps' tiles are one
+  const int tile = h->sf.ftile > 0 ? h->sf.ftile * (h->sf.fteam ? h->sf.fwpb : 1) : h->sf.tile;
+  *host_tile = (h->det || h->sf.fwpb == 0) ? 0 : tile;
   return DSMC_OK;
 }
 

@@ -261,13 +261,14 @@ class Dsmc:
         self._check(load().dsmc_synth_reuse(self._h, (1 if on else 0) | (2 if warm else 0)))
 
     def launch_config(self) -> int:
-        """Warps (cells) per CTA of the FP32 fused step chosen by the tuner."""
+        """Warps per CTA of the FP32 fused step chosen by the tuner."""
         v = ctypes.c_int()
         self._check(load().dsmc_get_launch_config(self._h, ctypes.byref(v)))
         return v.value
 
     def launch_shape(self) -> tuple:
-        """(warps per CTA, tile) of the FP32 fused step chosen by the tuner."""
+        """(warps per CTA, particles of a cell staged in shared memory) of the
+        FP32 fused step chosen by the tuner."""
         w, t = ctypes.c_int(), ctypes.c_int()
         self._check(load().dsmc_get_launch_shape(self._h, ctypes.byref(w), ctypes.byref(t)))
         return w.value, t.value
