@@ -82,54 +82,59 @@ __device__ void cta_exclusive_scan(int n, F value, int32_t* out) {
 }
 
 // ---------------------------------------------------------------------------
-// exclusive scan of v over the whole grid, CTA b the SCAN_CHUNK entries from b
-// SCAN_CHUNK: out[i] = sum_{k<i} v[k], out[n] = total.  A CTA adds up the
-// entries before its chunk itself (16-byte loads, from L2), so no CTA waits
-// for another and one launch does the scan; the redundant reads grow with
-// n^2 but are 13 MB at 160 000 cells.  Latency-bound; one CTA passing over
-// 160 000 cells in order took 107 us (three scans of a modification with
-// read-out of 32 M particles: 4.29 -> 3.99 ms in all).
+// exclusive scan of v over the whole grid, CTA b the `chunk` entries from b
+// chunk (a multiple of SCAN_PIECE): out[i] = sum_{k<i} v[k], out[n] = total.  A
+// CTA adds up the entries before its chunk itself (16-byte loads, from L2), so
+// no CTA waits for another and one launch does the scan.  At most a CTA per SM:
+// the redundant reads, half of n per CTA, then grow with n (13 MB at 160 000
+// cells) and not with n^2.  Latency-bound; one CTA passing over 160 000 cells in
+// order took 107 us (three scans of a modification with read-out of 32 M
+// particles: 4.29 -> 3.99 ms in all).  dsmc_num_particles of 16 M cells: 4.7 ms
+// with a CTA per 4 096 entries, 0.57 so; up to 622 592 cells both are the same.
 // total (may be null): the total is stored there too; flags (may be null):
 // bit 4 is set when the total exceeds capacity.
 // ---------------------------------------------------------------------------
-constexpr int SCAN_CHUNK = 4096;
-static __global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict__ v, int n, int32_t* __restrict__ out,
-                                                      int32_t* __restrict__ total, int32_t* __restrict__ flags,
-                                                      long long capacity) {
-  __shared__ int32_t s_pre[32], s_own[32];
+constexpr int SCAN_PIECE = 4096;
+static __global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict__ v, int n, int chunk,
+                                                      int32_t* __restrict__ out, int32_t* __restrict__ total,
+                                                      int32_t* __restrict__ flags, long long capacity) {
+  __shared__ int32_t s_pre[32], s_own[2][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int base = blockIdx.x * SCAN_CHUNK;
+  const int base = blockIdx.x * chunk, end = min(n, base + chunk);
   int32_t pre = 0;
   const int4* v4 = reinterpret_cast<const int4*>(v);
   for (int i = threadIdx.x; i < base / 4; i += 1024) {
     const int4 q = v4[i];
     pre += (q.x + q.y) + (q.z + q.w);
   }
-  const int i0 = base + 4 * (int)threadIdx.x;
-  int32_t e[4], t = 0;
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    e[j] = (i0 + j < n) ? v[i0 + j] : 0;
-    t += e[j];
-  }
-  int32_t x = t;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int32_t y = __shfl_up_sync(FULL, x, o);
-    if (lane >= o) x += y;
-  }
   pre = __reduce_add_sync(FULL, pre);
-  if (lane == 31) {
-    s_pre[warp] = pre;
-    s_own[warp] = x;
-  }
-  __syncthreads();
-  const int32_t before = __reduce_add_sync(FULL, s_pre[lane] + (lane < warp ? s_own[lane] : 0));
-  int32_t run = before + x - t;
+  if (lane == 0) s_pre[warp] = pre;
+  int32_t carry = 0, run = 0;
+  for (int p0 = base, k = 0; p0 < end; p0 += SCAN_PIECE, k ^= 1) {
+    const int i0 = p0 + 4 * (int)threadIdx.x;
+    int32_t e[4], t = 0;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    if (i0 + j < n) out[i0 + j] = run;
-    run += e[j];
+    for (int j = 0; j < 4; ++j) {
+      e[j] = (i0 + j < n) ? v[i0 + j] : 0;
+      t += e[j];
+    }
+    int32_t x = t;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int32_t y = __shfl_up_sync(FULL, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) s_own[k][warp] = x;
+    __syncthreads();  // two rows of s_own: the next piece's sums go to the other
+    if (p0 == base) carry = __reduce_add_sync(FULL, s_pre[lane]);
+    const int32_t own = s_own[k][lane];
+    run = carry + __reduce_add_sync(FULL, lane < warp ? own : 0) + x - t;
+    carry += __reduce_add_sync(FULL, own);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (i0 + j < n) out[i0 + j] = run;
+      run += e[j];
+    }
   }
   if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 1023) {
     out[n] = run;
@@ -140,7 +145,8 @@ static __global__ void __launch_bounds__(1024) k_scan(const int32_t* __restrict_
 
 inline void launch_scan(const int32_t* v, int n, int32_t* out, cudaStream_t st, int32_t* total = nullptr,
                         int32_t* flags = nullptr, long long capacity = 0) {
-  k_scan<<<(n + SCAN_CHUNK - 1) / SCAN_CHUNK, 1024, 0, st>>>(v, n, out, total, flags, capacity);
+  const int pieces = (n + SCAN_PIECE - 1) / SCAN_PIECE, per = (pieces + 151) / 152;
+  k_scan<<<(pieces + per - 1) / per, 1024, 0, st>>>(v, n, per * SCAN_PIECE, out, total, flags, capacity);
 }
 
 __device__ __forceinline__ int32_t bin_cap_of(int32_t count, double slack) {
