@@ -888,25 +888,21 @@ __device__ __forceinline__ void collide_cell(const Params<T>& p, T* __restrict__
 // ---------------------------------------------------------------------------
 //
 // FP32 particles: each step's sums go to Kahan-compensated FP32 staging
-// accumulators (stg, stc: 17 per cell; pre32 holds this lane's values loaded
-// earlier); when `flush` is set they are folded into the FP64 accumulators
-// and cleared.  FP64 particles add to the FP64 accumulators every step (pre
-// holds this lane's (acc, comp) loaded earlier, or is null).
-template <typename T>
-__device__ void sample_cell(const T* __restrict__ vx, const T* __restrict__ vy,
-                            const T* __restrict__ vz, const T* __restrict__ ir, int n,
-                            double* __restrict__ acc, double* __restrict__ comp,
-                            const double* pre = nullptr, float* __restrict__ stg = nullptr,
-                            float* __restrict__ stc = nullptr, const float* pre32 = nullptr,
-                            bool flush = true) {
+// accumulators (stg, stc: 17 per cell), which are folded into the FP64 ones
+// every few steps (sample_fold) and on a call's last step, here (pre32 holds
+// this lane's staged pair).  FP64 particles: sample_cell_f64.
+__device__ inline void sample_cell(const float* __restrict__ vx, const float* __restrict__ vy,
+                                   const float* __restrict__ vz, const float* __restrict__ ir, int n,
+                                   double* __restrict__ acc, double* __restrict__ comp, float* __restrict__ stg,
+                                   float* __restrict__ stc, const float* pre32) {
   const int lane = threadIdx.x & 31;
-  T s[NMOM];
+  float s[NMOM];
 #pragma unroll
-  for (int q = 0; q < NMOM; ++q) s[q] = T(0);
+  for (int q = 0; q < NMOM; ++q) s[q] = 0.f;
   for (int q = lane; q < n; q += 32) {
-    const T a = vx[q], b = vy[q], c = vz[q], e = ir[q];
-    const T v2 = a * a + b * b + c * c;
-    s[0] += T(1);
+    const float a = vx[q], b = vy[q], c = vz[q], e = ir[q];
+    const float v2 = a * a + b * b + c * c;
+    s[0] += 1.f;
     s[1] += a;
     s[2] += b;
     s[3] += c;
@@ -929,31 +925,20 @@ __device__ void sample_cell(const T* __restrict__ vx, const T* __restrict__ vy,
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(FULL, s[q], o);
   }
-  T mine = T(0);
+  float mine = 0.f;
 #pragma unroll
   for (int q = 0; q < NMOM; ++q)
     if (lane == q) mine = s[q];
   if (lane < NMOM) {
-    double v;
-    if (stg) {
-      // Kahan step into the FP32 staging pair
-      const float s0 = pre32[0], c0 = pre32[1];
-      const float yk = (float)mine - c0;
-      const float tk = s0 + yk;
-      const float ck = (tk - s0) - yk;
-      if (!flush) {
-        stg[lane] = tk;
-        stc[lane] = ck;
-        return;
-      }
-      stg[lane] = 0.f;
-      stc[lane] = 0.f;
-      v = (double)tk - (double)ck;
-    } else {
-      v = (double)mine;
-    }
-    const double a = pre ? pre[0] : acc[lane];
-    const double cprev = pre ? pre[1] : comp[lane];
+    // Kahan step into the FP32 staging pair, then the fold
+    const float s0 = pre32[0], c0 = pre32[1];
+    const float yk = mine - c0;
+    const float tk = s0 + yk;
+    const float ck = (tk - s0) - yk;
+    stg[lane] = 0.f;
+    stc[lane] = 0.f;
+    const double v = (double)tk - (double)ck;
+    const double a = acc[lane], cprev = comp[lane];
     const double t = a + v;
     const double cmp = (fabs(a) >= fabs(v)) ? ((a - t) + v) : ((v - t) + a);
     acc[lane] = t;

@@ -66,8 +66,8 @@ struct State {
   int32_t* start[2];  // layout: bin starts (ncells + 1) ...
   int32_t* count[2];  // ... and occupancies (ncells); those not in use are zero
   int32_t* cellof;    // FP64 compact layout: cell of each slot
-  int32_t* key;       // scratch: new cell per slot
-  int32_t* dest;      // scratch: destination slot
+  int32_t* key;       // scratch: new cell of each slot
+  int32_t* dest;      // scratch (FP64 layout): arrival number of each slot in its new cell
   int32_t* scratch_i; // scratch (capacity) for DIG index lists / export offsets
   uint32_t* owner;    // scratch (capacity) for the collision scheduler of big cells
   int32_t* nt;        // scratch (ncells): DIG target counts

@@ -25,7 +25,6 @@
 namespace dsmc {
 
 constexpr int WPB = 8;  // warps per CTA for the per-cell kernels
-constexpr int CTA_SCAN = 1024;
 
 // ---------------------------------------------------------------------------
 // single-CTA exclusive scan: out[i] = sum_{k<i} value(k), out[n] = total
@@ -859,19 +858,20 @@ __global__ void __launch_bounds__(WPB * 32) k_det_cells(const __grid_constant__ 
 
 // One warp per cell: stage the cell's velocities and rotational energies in
 // shared memory (cells above `tile` particles work in global memory), run
-// NTC collisions and/or sampling, write back.  flags: 1 collide, 2 sample.
-template <typename T, bool BATCH>
-__global__ void __launch_bounds__(WPB * 32) k_collide_sample(const __grid_constant__ Params<T> pk, Cases<T> cases,
-                                                             int ncells, PBuf<T> b,
+// NTC collisions and/or sampling, write back: the last step of a call in the
+// FP32 layout, which has no move behind it.  flags: 1 collide, 2 sample.
+template <bool BATCH>
+__global__ void __launch_bounds__(WPB * 32) k_collide_sample(const __grid_constant__ Params<float> pk,
+                                                             Cases<float> cases, int ncells, PBuf<float> b,
                                                              const int32_t* __restrict__ start,
                                                              const int32_t* __restrict__ count,
-                                                             T* __restrict__ sgmax, double* __restrict__ acc,
+                                                             float* __restrict__ sgmax, double* __restrict__ acc,
                                                              double* __restrict__ comp,
                                                              uint32_t* __restrict__ owner_g,
                                                              uint32_t step, int flags, int tile,
                                                              unsigned long long* __restrict__ stats,
-                                                             float* __restrict__ stg = nullptr,
-                                                             float* __restrict__ stc = nullptr) {
+                                                             float* __restrict__ stg,
+                                                             float* __restrict__ stc) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ unsigned s_cnt[4];
   if (threadIdx.x < 4) s_cnt[threadIdx.x] = 0;
@@ -880,13 +880,13 @@ __global__ void __launch_bounds__(WPB * 32) k_collide_sample(const __grid_consta
   const int cell = blockIdx.x * WPB + warp;
   if (cell < ncells) {
     const int cs = BATCH ? cases.cell_case[cell] : 0;
-    const Params<T>& p = BATCH ? cases.p[cs] : pk;
+    const Params<float>& p = BATCH ? cases.p[cs] : pk;
     const int lcell = cell - (BATCH ? cases.cell0[cs] : 0);
     const int base = start[cell], n = count[cell];
-    T* tv = reinterpret_cast<T*>(smem) + (size_t)warp * tile * 4;
-    uint32_t* tow = reinterpret_cast<uint32_t*>(smem + (size_t)WPB * tile * 4 * sizeof(T)) + (size_t)warp * tile;
+    float* tv = reinterpret_cast<float*>(smem) + (size_t)warp * tile * 4;
+    uint32_t* tow = reinterpret_cast<uint32_t*>(smem + (size_t)WPB * tile * 4 * sizeof(float)) + (size_t)warp * tile;
     const bool staged = n <= tile;
-    T *vx, *vy, *vz, *ir;
+    float *vx, *vy, *vz, *ir;
     uint32_t* own;
     if (staged) {
       vx = tv;
@@ -910,23 +910,18 @@ __global__ void __launch_bounds__(WPB * 32) k_collide_sample(const __grid_consta
     __syncwarp();
     if (flags & 1) {
       CollCount cc{0, 0, 0, 0};
-      collide_cell<T>(p, vx, vy, vz, ir, n, (uint32_t)lcell, step, sgmax + cell, own, cc);
-      flush_counts<T>(cc, s_cnt);
+      collide_cell<float>(p, vx, vy, vz, ir, n, (uint32_t)lcell, step, sgmax + cell, own, cc);
+      flush_counts<float>(cc, s_cnt);
       __syncwarp();
     }
     if (flags & 2) {
-      if (stg) {
-        // FP32 staging accumulators: always folded here (last step of a call)
-        float pre32[2] = {0.f, 0.f};
-        if (lane < NMOM) {
-          pre32[0] = stg[(size_t)cell * NMOM + lane];
-          pre32[1] = stc[(size_t)cell * NMOM + lane];
-        }
-        sample_cell<T>(vx, vy, vz, ir, n, acc + (size_t)cell * NMOM, comp + (size_t)cell * NMOM, nullptr,
-                       stg + (size_t)cell * NMOM, stc + (size_t)cell * NMOM, pre32, true);
-      } else {
-        sample_cell<T>(vx, vy, vz, ir, n, acc + (size_t)cell * NMOM, comp + (size_t)cell * NMOM);
+      float pre32[2] = {0.f, 0.f};
+      if (lane < NMOM) {
+        pre32[0] = stg[(size_t)cell * NMOM + lane];
+        pre32[1] = stc[(size_t)cell * NMOM + lane];
       }
+      sample_cell(vx, vy, vz, ir, n, acc + (size_t)cell * NMOM, comp + (size_t)cell * NMOM,
+                  stg + (size_t)cell * NMOM, stc + (size_t)cell * NMOM, pre32);
     }
     if (staged && (flags & 1)) {
       for (int q = lane; q < n; q += 32) {
@@ -2344,15 +2339,6 @@ static size_t tile_smem(int tile) {
   return (size_t)WPB * tile * (4 * sizeof(T) + sizeof(uint32_t));
 }
 
-template <typename T, bool BATCH>
-static void launch_collide_sample(const Params<T>& p, State<T>& s, int ncells, const PBuf<T>& b, const int32_t* start,
-                                  const int32_t* count, uint32_t step, int flags, float* stg, float* stc,
-                                  cudaStream_t st) {
-  const int blocks = (ncells + WPB - 1) / WPB;
-  k_collide_sample<T, BATCH><<<blocks, WPB * 32, tile_smem<T>(s.tile), st>>>(
-      p, s.cases, ncells, b, start, count, s.sgmax, s.acc, s.comp, s.owner, step, flags, s.tile, s.stats, stg, stc);
-}
-
 // up to this many slots and cells: scan and lists in one single-CTA launch
 // (one launch less, about 3 us, where a CTA's 1024 threads take at most 16
 // slots each).  A step of 10 000 particles on 100 cells: 138 us with the
@@ -2453,13 +2439,9 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
   p, s.cases, ncells, s.buf[cur], s.buf[other], s.start[lay], s.count[cur], s.count[other], s.sgmax, s.acc,        \
       s.comp, s.ovf[cur], s.ovf[other], s.ovf_cap, s.ovf_spare, sc, sm_step, flags, ftile, cblocks, s.tally,       \
       s.stats, s.flags + 8, s.stg, s.stc
-#define DSMC_TEAM_ARGS                                                                                            \
-  p, s.cases, ncells, s.buf[cur], s.buf[other], s.start[lay], s.count[cur], s.count[other], s.sgmax, s.acc,        \
-      s.comp, s.ovf[cur], s.ovf[other], s.ovf_cap, s.ovf_spare, sc, sm_step, flags, ftile, cblocks, s.tally,       \
-      s.stats, s.flags + 8, s.stg, s.stc
 #define DSMC_FUSED_LAUNCH(D, B, W, A)                                                      \
   launch_pdl(!A, k_fused<D, B, W, A, false>, blocks, W * 32, smf, st, DSMC_FUSED_ARGS)
-#define DSMC_TEAM_LAUNCH(D, B) launch_pdl(true, k_fused_team<D, B>, blocks, TEAM_WARPS * 32, smf, st, DSMC_TEAM_ARGS)
+#define DSMC_TEAM_LAUNCH(D, B) launch_pdl(true, k_fused_team<D, B>, blocks, TEAM_WARPS * 32, smf, st, DSMC_FUSED_ARGS)
 #define DSMC_FUSED_LAUNCH_GEN(D, A) \
   launch_pdl(!A, k_fused<D, false, 4, A, true>, blocks, 128, smf, st, DSMC_FUSED_ARGS)
       const bool inject = p.mesh == 1;
@@ -2510,7 +2492,6 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
       }
 #undef DSMC_FUSED_LAUNCH
 #undef DSMC_TEAM_LAUNCH
-#undef DSMC_TEAM_ARGS
 #undef DSMC_FUSED_LAUNCH_GEN
 #undef DSMC_FUSED_ARGS
       if (inject) cudaStreamWaitEvent(st, s.ev_join, 0);
@@ -2578,12 +2559,10 @@ void Ops<T>::step_bins(const Params<T>& p, State<T>& s, int& cur, int lay, uint3
         launch(fused_flags(i), sc, sc + 1, F, FT, s.fteam);
       } else {
         const int flags = 1 | (do_sample ? 2 : 0);
-        if (s.batch)
-          launch_collide_sample<T, true>(p, s, ncells, s.buf[cur], s.start[lay], s.count[cur], sc, flags, s.stg,
-                                         s.stc, st);
-        else
-          launch_collide_sample<T, false>(p, s, ncells, s.buf[cur], s.start[lay], s.count[cur], sc, flags, s.stg,
-                                          s.stc, st);
+        auto* kern = s.batch ? k_collide_sample<true> : k_collide_sample<false>;
+        kern<<<(ncells + WPB - 1) / WPB, WPB * 32, tile_smem<T>(s.tile), st>>>(
+            p, s.cases, ncells, s.buf[cur], s.start[lay], s.count[cur], s.sgmax, s.acc, s.comp, s.owner, sc, flags,
+            s.tile, s.stats, s.stg, s.stc);
       }
     }
   } else {
@@ -2746,8 +2725,8 @@ void Ops<T>::configure(int tile) {
     cudaFuncSetAttribute(k_det_cells<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
     cudaFuncSetAttribute(k_det_cells<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   } else {
-    cudaFuncSetAttribute(k_collide_sample<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
-    cudaFuncSetAttribute(k_collide_sample<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(k_collide_sample<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    cudaFuncSetAttribute(k_collide_sample<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
   }
   if constexpr (sizeof(T) == 4) {
     const int smt = (int)fused_smem_bytes(tile, TEAM_WARPS);

@@ -466,13 +466,16 @@ __global__ void __launch_bounds__(S2_NT) k_s2_trail(const s2::Grid g, S2Work w, 
 // memory at once, each row's multipliers to shared memory (Ls, by load
 // index) until the end, when they are stored at the rows' final positions.
 // The pivots are chosen as in k_s2_panel (largest magnitude, lowest position
-// among equals), and each entry takes the same operations in the same order.
+// among equals), and within the panel each entry takes the same operations in
+// the same order.
 //
 // One launch does the panel at k0 and what is left of the panel before it
 // (kp = k0 - 32; none: kp < 0): CTA 0 applies that one to its own 32 columns
 // as it loads them (interchanges by where a row is read from; the rank-32
-// update row by row in registers), the other CTAs to the columns beyond,
-// cbt each.  So the panels' chain does not wait for the trailing columns.
+// update in registers as 32 subtractions, where s2::trail_l21 subtracts one sum
+// of 32 products: the factors differ in FP32 rounding, which the refinement
+// takes up), the other CTAs to the columns beyond, cbt each.  So the panels'
+// chain does not wait for the trailing columns.
 // 100 x 100 (1 036 rows): 52 us a panel and 23 us its trailing columns as two
 // launches, 57 us as one.  A column's chain of steps over the warps bounds it
 // (barrier, pivot row, division, update, search), not issue.
