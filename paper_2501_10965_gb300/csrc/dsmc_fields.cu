@@ -869,7 +869,7 @@ static cudaError_t run_synth(const SynthCases& sc, const int32_t* host_nx, doubl
   // more slabs than two per SM: half the threads per slab, so that an SM holds
   // twice the slabs (the kernels use up to 128 registers a thread) and their
   // FP64 phases and reduction levels overlap (800 slabs of 200 cells, a fresh
-  // solve: 1.28 ms with 256 threads, 1.23 ms with 128; up to two slabs per SM
+  // solve: 1.29 ms with 256 threads, 1.25 ms with 128; up to two slabs per SM
   // are resident at once either way, and fewer threads only lengthen each)
   if (sc.ncases > 2 * 152) nmax = (nmax + 1) / 2;
   if (nmax <= 128) return run_synth_nt<128>(sc, out, n_m, tol, st);

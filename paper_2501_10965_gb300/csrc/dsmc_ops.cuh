@@ -716,10 +716,13 @@ __device__ __forceinline__ void gather_cell(const int32_t* __restrict__ order, i
 // The FP64 pipe bounds it (one warp instruction per 16 cycles and SM, however
 // many lanes are active) and a cell has few candidates, so with 8 warps per
 // CTA one warp takes the candidates of four cells, 8 lanes each, when none of
-// them has more than GROUP_MAX_M: a quarter of the instructions.  GROUP_MAX_M:
-// above it the 8-lane window's rounds outnumber what the sharing saves.  With
-// one warp per CTA (few cells: every cell has an SM's pipe to itself) the
-// cell's own warp takes them.
+// them has more than GROUP_MAX_M: a quarter of the instructions.  GROUP_MAX_M
+// keeps an 8-lane group's rounds few where the cells leave SMs idle and a step
+// lasts as long as one cell's chain: 900 cells of 50 particles, 12 candidates a
+// cell 76 us a step grouped and 88 not, 24 115 and 129, 49 205 and 207.  With
+// the SMs full the line is lower than it need be: 10 000 cells, 12 candidates
+// 262 and 484 us, 24 411 and 766, 49 726 and 1 321.  With one warp per CTA (few
+// cells: every cell has an SM's pipe to itself) the cell's own warp takes them.
 constexpr uint32_t GROUP_MAX_M = 24u;
 template <typename T, bool BATCH>
 __global__ void __launch_bounds__(WPB * 32) k_det_cells(const __grid_constant__ Params<T> pk, Cases<T> cases,
